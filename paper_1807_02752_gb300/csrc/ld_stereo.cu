@@ -3,17 +3,13 @@
 // disparity map, then the left-right consistency check (Alg. 3).  Kernels and the ld_stereo_* entry
 // points of include/ld.h.
 //
-//   k_srp   one CTA per (frame, map): rows from H-1-rho up to rho, in order, since a row's search range
-//           comes from the row below.  A ring of the 2 rho + 1 image rows of both images sits in shared
-//           memory, stored by column (a column's rows in 8 bytes); when the window moves up one row the new
-//           top row (loaded a row ahead) replaces the old bottom row and per-column sums of I and I^2 are
-//           updated by their difference, so the block statistics of every pixel of the row are two 7-wide
-//           sums of column sums (exact integers, the quantities the paper gets from integral images, Eq. 5).
-//           A thread takes a pixel, keeps its block's columns in registers and forms each candidate's
-//           block product P from 7 column dot products (two dp4a each, in four independent chains).  The best candidate has the
-//           largest NCC, compared exactly: c = N / sqrt(D_a D_b) with N = n P - s_a s_b and
-//           D = n Q - s^2, so c1 > c2 <=> N1 |N1| D2 > N2 |N2| D1 (a float filter decides clear cases,
-//           128-bit integers the rest).
+//   k_srp   one CTA, or one cluster of CTAs that share a row, per (frame, map): rows from H-1-rho up to rho,
+//           in order, since a row's search range comes from the row below (the layout is described at the
+//           kernel).  The best candidate has the largest NCC, compared exactly: c = N / sqrt(D_a D_b) with
+//           N = n P - s_a s_b and D = n Q - s^2 (s, Q, P: block sums of I, I^2 and the product, exact
+//           integers, the quantities the paper gets from integral images, Eq. 5), so
+//           c1 > c2 <=> N1 |N1| D2 > N2 |N2| D1 (a float filter decides clear cases, 128-bit integers the
+//           rest).
 //   k_lrc   l(u, v) = l_lf(u, v) when |l_lf(u, v) - l_rt(u - l_lf(u, v), v)| <= tr, else 0; float output.
 //
 // Readings: blocks lie inside both images (other pixels and candidates are skipped; a pixel without a
@@ -28,246 +24,621 @@ namespace ld {
 
 namespace {
 
-constexpr int kSrpThreads = 512;
-
 struct SrpArgs {
     const uint8_t *left, *right;     // [n][H][W]
     int16_t *lf, *rt;                // [n][H][W]
     int W, H, dmax, tau;
+    // launch shape (SrpShape)
+    int per;                         // pixels a CTA of the cluster owns
+    int strips, n_extra;             // its strips, and those of the other image beyond them
+    int groups;                      // warps that search a strip (the first strips x groups warps of a CTA)
 };
 
-// c1 > c2 for c = N / sqrt(D) (a common positive factor dropped); D = 0 means c = 0.  Decided exactly:
-// c1 > c2 <=> N1 |N1| D2 > N2 |N2| D1.  Each side in float carries four roundings (the two conversions and
-// two products; relative error about 2^-22), so a float gap above 2^-20 (|L| + |R|) has the sign of the
-// exact one; closer pairs compare in 128-bit integers.
-__device__ __forceinline__ bool ncc_better(long long N1, int D1, long long N2, int D2)
+constexpr int kSrpMaxWarps = 24;     // warps of a CTA (80 registers a thread)
+constexpr int kSrpFewWarps = 16;     // ... of the variant with 128 registers, for the CTAs of few pairs
+constexpr int kSrpPrep = 4;          // strips of the other image a preparing warp takes at most
+constexpr int kSrpShared = 12;       // distinct disparities up to which a strip walks their union in any case
+constexpr int kSrpHalo = 8;          // rows between two exchanges of a cluster = halo pixels on each side
+
+// Pixels of a strip: a warp's 64 columns less the 2 rho that only complete the blocks of its neighbours.
+__host__ __device__ constexpr int srp_strip(int rho) { return 64 - 2 * rho; }
+// Entries of one buffer of the other image (16 bytes each).
+__host__ __device__ inline int srp_entries(int warps, int n_extra, int rho)
 {
-    if (D1 == 0)
-        N1 = 0;
-    if (D2 == 0)
-        N2 = 0;
-    if (N1 == 0 || N2 == 0)
-        return N2 == 0 ? N1 > 0 : N2 < 0 && N1 == 0;
-    const float f1 = (float)N1, f2 = (float)N2;
-    const float L = __fmul_rn(__fmul_rn(f1, fabsf(f1)), (float)D2);
-    const float R = __fmul_rn(__fmul_rn(f2, fabsf(f2)), (float)D1);
-    const float gap = __fsub_rn(L, R);
-    if (fabsf(gap) > 9.5367431640625e-07f * (fabsf(L) + fabsf(R)))
-        return gap > 0.0f;
-    const __int128 l = (__int128)N1 * (N1 < 0 ? -N1 : N1) * D2;
-    const __int128 r = (__int128)N2 * (N2 < 0 ? -N2 : N2) * D1;
-    return l > r;
+    return srp_strip(rho) * (warps + n_extra) + 2 * rho;
 }
 
-constexpr int kMaxColsPerThread = 8;  // columns per thread in the row loads (the launch guarantees W <= 8 x threads)
-
-// threads of a k_srp CTA: the pixels with a block spread evenly (every thread the same number of them),
-// at most kSrpThreads, and enough threads that each loads at most kMaxColsPerThread columns of a row
-inline int srp_threads(int W, int rho)
+__device__ __forceinline__ uint32_t srp_shl(uint32_t x, int n)   // 0 for n >= 32
 {
-    const int valid = W - 2 * rho, per = (valid + kSrpThreads - 1) / kSrpThreads;
-    int t = (valid + per - 1) / per;
-    t = t > (W + kMaxColsPerThread - 1) / kMaxColsPerThread ? t : (W + kMaxColsPerThread - 1) / kMaxColsPerThread;
-    t = t < 32 ? 32 : t;
-    return t < kSrpThreads ? t : kSrpThreads;
+    uint32_t r;
+    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(n));
+    return r;
+}
+// Bits b of [0, 32) with lo <= b <= hi.
+__device__ __forceinline__ uint32_t srp_bits(int lo, int hi)
+{
+    return srp_shl(0xffffffffu, max(lo, 0)) & ~srp_shl(0xffffffffu, max(hi + 1, 0));
+}
+__device__ __forceinline__ float srp_rsqrt(float x)   // x >= 1; relative error at most 2^-22.9
+{
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ uint4 srp_lds(uint32_t a)
+{
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ uint2 srp_lds2(uint32_t a)
+{
+    uint2 v;
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ void cluster_sync_all()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// A lane's two adjacent image columns: the K rows of the block window in K bytes (the newest in byte 0) and
+// the window's sums of I and I^2.
 template <int RHO>
-__global__ void __launch_bounds__(kSrpThreads, 1) k_srp(const SrpArgs a)
+struct SrpCols {
+    uint32_t lo[2], hi[2];
+    int s[2], q[2];
+    __device__ __forceinline__ void push(int c, int x)   // the row above enters, the bottom row leaves
+    {
+        constexpr int K = 2 * RHO + 1;
+        int old;
+        if constexpr (K > 4) {
+            old = (int)(hi[c] >> (8 * (K - 5)));
+            hi[c] = __funnelshift_l(lo[c], hi[c], 8) & ((1u << (8 * (K - 4))) - 1u);
+            lo[c] = (lo[c] << 8) | (uint32_t)x;
+        } else {
+            old = (int)(lo[c] >> (8 * (K - 1)));
+            lo[c] = ((lo[c] << 8) | (uint32_t)x) & ((1u << (8 * K)) - 1u);
+        }
+        s[c] += x - old;
+        q[c] += (x - old) * (x + old);
+    }
+};
+
+// Sums over the K columns of the blocks of a lane's two pixels (leftmost columns 2 lane and 2 lane + 1 of
+// the strip), for N quantities at once, from the per-column values c0, c1: sum_1 = c1 + sum_{k = 1 .. rho}
+// (c0 + c1) of lane + k, and sum_0 differs by the outer columns.  Valid on lanes below srp_strip / 2.  The N
+// chains go through each shuffle together (shuffles keep their order, so one chain after the other would
+// wait out every latency).
+template <int RHO, int N>
+__device__ __forceinline__ void srp_block_sums(const int *c0, const int *c1, int *p0, int *p1)
 {
-    constexpr int K = 2 * RHO + 1, NB = K * K;
+    constexpr unsigned kAll = 0xffffffffu;
+    int t1[N], last[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+        t1[k] = __shfl_down_sync(kAll, c0[k] + c1[k], 1);
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+        last[k] = __shfl_down_sync(kAll, c1[k], RHO);
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        if constexpr (RHO == 1)
+            p1[k] = c1[k] + t1[k];
+        else if constexpr (RHO == 2)
+            p1[k] = c1[k] + t1[k] + __shfl_down_sync(kAll, c0[k] + c1[k], 2);
+        else
+            p1[k] = c1[k] + t1[k] + __shfl_down_sync(kAll, c0[k] + c1[k] + t1[k], 2);
+    }
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+        p0[k] = p1[k] + c0[k] - last[k];
+}
+
+// N and D_B of the blocks of A around (u, v) and of B around (ub, v), from the images.
+template <int RHO>
+__device__ void srp_block_nd(const uint8_t *A, const uint8_t *B, int W, int v, int u, int ub, long long &N, long long &D)
+{
+    constexpr int NB = (2 * RHO + 1) * (2 * RHO + 1);
+    int P = 0, sa = 0, sb = 0, Q = 0;
+    for (int y = -RHO; y <= RHO; ++y)
+        for (int x = -RHO; x <= RHO; ++x) {
+            const int g = A[(size_t)(v + y) * W + u + x], h = B[(size_t)(v + y) * W + ub + x];
+            P += g * h;
+            sa += g;
+            sb += h;
+            Q += h * h;
+        }
+    N = NB * P - sa * sb;
+    D = NB * Q - sb * sb;
+}
+
+// The best candidate of pixel (u, v) by exact comparison, for the rare pixel whose two best float scores are
+// too close: candidates are the d <= dhi within t of l0, l1 or l2, ascending; c1 > c2 <=>
+// N1 |N1| D2 > N2 |N2| D1, and c = 0 where a block is constant (then N = 0).
+template <int RHO>
+__device__ __noinline__ int srp_exact_best(const uint8_t *A, const uint8_t *B, int W, int v, int u, int sign, int l0,
+                                           int l1, int l2, int t, int dhi)
+{
+    int best = -1;
+    long long bN = 0, bD = 0;
+    for (int d = max(min(min(l0, l1), l2) - t, 0); d <= min(max(max(l0, l1), l2) + t, dhi); ++d) {
+        if (abs(d - l0) > t && abs(d - l1) > t && abs(d - l2) > t)
+            continue;
+        long long N, D;
+        srp_block_nd<RHO>(A, B, W, v, u, u + sign * d, N, D);
+        bool better = best < 0;
+        if (!better) {
+            if (N == 0 || bN == 0)
+                better = N > bN;
+            else
+                better = (__int128)(N * (N < 0 ? -N : N)) * bD > (__int128)(bN * (bN < 0 ? -bN : bN)) * D;
+        }
+        if (better) {
+            best = d;
+            bN = N;
+            bD = D;
+        }
+    }
+    return best;
+}
+
+// Layout.  A warp owns a strip of 64 image columns, two adjacent ones per lane, and the 64 - 2 rho pixels
+// whose blocks they complete.  Column dot products (two dp4a) of the strip with the other image at one
+// disparity d give the block products P of all its pixels through three shuffles, instead of 2 rho + 1
+// column products per pixel and candidate: neighbouring pixels mostly search the same few disparities (the
+// rows of the synthetic pairs need 6 to 10 distinct ones per strip and row, and 3.3 to 3.8 per pixel), so
+// the warp walks the union of its pixels' search ranges, 32 disparities at a time as a bit mask, and each
+// pixel takes part at its own candidates.  A lane keeps its columns of image A and their sums in registers
+// (the window moves up a row by a byte shift) and publishes the same of image B in shared memory, one
+// 16-byte entry per column {rows 0-3, rows 4-6, s_B, 1 / sqrt(D_B)}, even and odd columns apart so that a
+// warp's loads of any d are contiguous; double-buffered by row, so one barrier per row suffices.
+// N and D fit 32 bits (n^2 255^2 < 2^28).  The score N / sqrt(D_B) is a float: the conversions, the product
+// and rsqrt.approx (relative error 2^-22.9) err by less than 2^-21 together, so when the best score leads
+// the second best by more than 2^-20 (|s1| + |s2|) the best candidate is the exact one; otherwise the pixel's
+// candidates are compared again in integers, from the images (about one pixel in 10^4).  Ascending d and a
+// strict comparison give ties to the smaller disparity.
+//
+// Few pairs leave most SMs idle, so a map's columns are then split over a cluster (CLUSTER): each CTA also
+// computes kSrpHalo pixels beyond its own on either side, which a pixel per row becomes stale (a row reads
+// its neighbours' estimates one pixel away); every kSrpHalo rows the CTAs write their edge estimates into
+// the neighbours' shared memory and meet at a cluster barrier.  A CTA then has few strips, and the row is a
+// chain of latencies: one or two warps search a strip (two take the even and the odd disparities and merge
+// through shared memory) and others prepare the other image, NPREP strips each.  With a whole map per CTA
+// the strips' own warps do both.
+//
+// What bounds it: the rows follow one another (369 at 1242x375).  One CTA per map: the ALU pipe (two cycles
+// per integer instruction) and the wait for the strip with the most distinct disparities.  Clusters: the
+// latency chain of a row (about 4400 cycles).  At 1242x375, d_max 127: 64 pairs 3.42 -> 1.83 ms, one pair
+// 3.19 -> 0.76 ms, against every pixel forming its own candidates' products with one CTA per map.
+template <int RHO, int NPREP, bool CLUSTER, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, 1) k_srp(const SrpArgs a)
+{
+    constexpr int S = srp_strip(RHO), K = 2 * RHO + 1, NB = K * K;
+    constexpr int kWin = 30;          // disparities of one candidate mask
+    constexpr int kBatch = CLUSTER ? 2 : 3;   // disparities of the union in flight together
     extern __shared__ __align__(16) unsigned char sm[];
-    const int W = a.W, H = a.H, f = blockIdx.x, dir = blockIdx.y;
+    const int W = a.W, H = a.H, f = blockIdx.y, dir = blockIdx.z, rank = blockIdx.x, nrank = gridDim.x;
     const size_t fo = (size_t)f * H * W;
     const uint8_t *A = (dir == 0 ? a.left : a.right) + fo;   // the image whose map this is
     const uint8_t *B = (dir == 0 ? a.right : a.left) + fo;
     int16_t *out = (dir == 0 ? a.lf : a.rt) + fo;
-    // ring of the K block rows, stored by column: byte r of column c is ring slot r (row y with y % K == r),
-    // byte 7 stays 0, so the dot product of two columns is two dp4a
-    uint2 *ca = reinterpret_cast<uint2 *>(sm);                 // [W]
-    uint2 *cb = ca + W;                                        // [W]
-    int *cs = reinterpret_cast<int *>(cb + W);                 // [4][W]: column sums of A, A^2, B, B^2
-    int2 *ra2 = reinterpret_cast<int2 *>(cs + 4 * W);           // [W]: block (s_A, D_A) of the row
-    int2 *rb2 = ra2 + W;                                       // [W]: block (s_B, D_B)
-    int16_t *lv = reinterpret_cast<int16_t *>(rb2 + W);        // [2][W]: estimates of the row below / this row
-    uint8_t *ca8 = reinterpret_cast<uint8_t *>(ca), *cb8 = reinterpret_cast<uint8_t *>(cb);
-    const int tid = threadIdx.x, nthr = blockDim.x;
-    const int vb = H - 1 - RHO;
-    for (int i = tid; i < RHO * W; i += nthr) {
-        out[i] = 0;
-        out[(size_t)(H - RHO) * W + i] = 0;
-    }
-    // initial window: rows vb - RHO .. vb + RHO
-    for (int u = tid; u < W; u += nthr) {
-        int s0 = 0, q0 = 0, s1 = 0, q1 = 0;
-        uint8_t xa[8], xb[8];
-#pragma unroll
-        for (int r = 0; r < 8; ++r)
-            xa[r] = xb[r] = 0;
-        for (int y = vb - RHO; y <= vb + RHO; ++y) {
-            const int x = A[(size_t)y * W + u], z = B[(size_t)y * W + u];
-            xa[y % K] = (uint8_t)x;
-            xb[y % K] = (uint8_t)z;
-            s0 += x;
-            q0 += x * x;
-            s1 += z;
-            q1 += z * z;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = a.strips;
+    const int n_search = nw * a.groups, group = warp / nw;   // searching warps: strip warp % nw, group warp / nw
+    const bool search = !CLUSTER || warp < n_search;
+    const int strip = warp - group * nw;
+    const int vb = H - 1 - RHO, umax = W - 1 - RHO;
+    const int own0 = RHO + rank * a.per, own1 = min(own0 + a.per, W - RHO);   // pixels [own0, own1)
+    const int px0 = own0 - (CLUSTER && rank > 0 ? kSrpHalo : 0);              // first pixel computed
+    const int col0 = px0 - RHO;                                               // its leftmost column
+    const int ent0 = col0 - (dir == 0 ? S * a.n_extra : 0);                   // column of entry 0
+    const int n_ent = srp_entries(nw, a.n_extra, RHO);
+    const uint32_t odd = 16u * (uint32_t)(n_ent >> 1), buf_bytes = 2u * odd;
+    const uint32_t ent = (uint32_t)__cvta_generic_to_shared(sm);
+    // estimates of the row below and of this row: two int16 per pair of pixels, a missing pair before the
+    // first and after the last
+    uint32_t *lv = reinterpret_cast<uint32_t *>(sm + 2 * (size_t)buf_bytes);   // [2][nw S / 2 + 2]
+    const int n_lv = nw * (S / 2) + 2;
+    int16_t *inbox = reinterpret_cast<int16_t *>(lv + 2 * n_lv);               // [2][2 kSrpHalo] left, right halo
+    float *half = reinterpret_cast<float *>(inbox + 4 * kSrpHalo);             // [6][32 nw] second group's bests
+
+    const int pair = strip * (S / 2) + lane;              // the lane's pair of pixels px0 + 2 pair, + 1
+    const int u0 = px0 + 2 * pair;
+    const bool mine = lane < S / 2;
+    const bool in0 = search && mine && u0 <= umax, in1 = search && mine && u0 + 1 <= umax;
+    const bool st0 = in0 && group == 0 && u0 >= own0 && u0 < own1, st1 = in1 && group == 0 && u0 + 1 >= own0 && u0 + 1 < own1;
+    int dhi0 = dir == 0 ? u0 - RHO : umax - u0, dhi1 = dir == 0 ? u0 + 1 - RHO : umax - u0 - 1;
+    dhi0 = in0 ? min(dhi0, a.dmax) : -1;
+    dhi1 = in1 ? min(dhi1, a.dmax) : -1;
+
+    // borders without a block: rows by the first CTA of the cluster, columns likewise
+    if (rank == 0) {
+        for (int i = tid; i < RHO * W; i += blockDim.x) {
+            out[i] = 0;
+            out[(size_t)(H - RHO) * W + i] = 0;
         }
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            ca8[u * 8 + r] = xa[r];
-            cb8[u * 8 + r] = xb[r];
+        for (int i = tid; i < (H - 2 * RHO) * 2 * RHO; i += blockDim.x) {
+            const int r = i / (2 * RHO), c = i - r * 2 * RHO;
+            out[(size_t)(RHO + r) * W + (c < RHO ? c : W - 2 * RHO + c)] = 0;
         }
-        cs[u] = s0;
-        cs[W + u] = q0;
-        cs[2 * W + u] = s1;
-        cs[3 * W + u] = q1;
     }
-    // the row entering next (vb - RHO - 1), loaded a row ahead
-    int na[kMaxColsPerThread], nb[kMaxColsPerThread];
+    for (int i = tid; i < 2 * n_lv; i += blockDim.x)
+        lv[i] = 0xffffffffu;   // -1: no estimate
+
+    // strips of B this warp prepares (counted from column ent0): its own, or a preparing warp's share
+    int bcol[NPREP];
+    bool bon[NPREP];
+    const int n_prep = (int)(blockDim.x >> 5) - n_search;
 #pragma unroll
-    for (int k = 0; k < kMaxColsPerThread; ++k) {
-        const int u = tid + k * nthr, y = vb - RHO - 1;
-        na[k] = (u < W && y >= 0) ? A[(size_t)y * W + u] : 0;
-        nb[k] = (u < W && y >= 0) ? B[(size_t)y * W + u] : 0;
+    for (int k = 0; k < NPREP; ++k) {
+        const int at = warp - n_search + k * n_prep;
+        bcol[k] = CLUSTER ? ent0 + S * at : col0 + S * strip;
+        bon[k] = (CLUSTER ? !search && at < nw + a.n_extra : true) && bcol[k] < W && bcol[k] + 64 > 0;
     }
-    int cur = 0;
+    const int bend = CLUSTER ? ent0 + S * (nw + a.n_extra) : col0 + S * nw;   // first column no strip begins at
+    // row y of the lane's two columns (the caller's pointer to them); columns off the image read 0
+    auto load2 = [&](const uint8_t *p, int c, bool on, int *x) {
+        x[0] = on && c >= 0 && c < W ? (int)__ldg(p) : 0;
+        x[1] = on && c >= -1 && c < W - 1 ? (int)__ldg(p + 1) : 0;
+    };
+    const int acol = col0 + 2 * pair;
+    const uint8_t *pa = A + (ptrdiff_t)(vb + RHO) * W + acol, *pb[NPREP];
+#pragma unroll
+    for (int k = 0; k < NPREP; ++k)
+        pb[k] = B + (ptrdiff_t)(vb + RHO) * W + bcol[k] + 2 * lane;
+    SrpCols<RHO> ac = {}, bc[NPREP] = {};
+    int sa0 = 0, sa1 = 0;
+    auto publish = [&](int k, uint32_t to) {
+        const int c0[2] = {bc[k].s[0], bc[k].q[0]}, c1[2] = {bc[k].s[1], bc[k].q[1]};
+        int p0[2], p1[2];
+        srp_block_sums<RHO, 2>(c0, c1, p0, p1);
+        const int s0 = p0[0], q0 = p0[1], s1 = p1[0], q1 = p1[1];
+        const int D0 = NB * q0 - s0 * s0, D1 = NB * q1 - s1 * s1;
+        const float i0 = D0 > 0 ? srp_rsqrt((float)D0) : 0.0f, i1 = D1 > 0 ? srp_rsqrt((float)D1) : 0.0f;
+        const int next = bcol[k] + S;   // the next strip is prepared when it holds columns of the image
+        const bool all = next >= W || next >= bend;
+        if (mine || all) {
+            const uint32_t at = to + 16u * (uint32_t)(((bcol[k] - ent0) >> 1) + lane);
+            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(bc[k].lo[0]), "r"(bc[k].hi[0]),
+                         "r"(s0), "r"(__float_as_int(i0)) : "memory");
+            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(at + odd), "r"(bc[k].lo[1]), "r"(bc[k].hi[1]),
+                         "r"(s1), "r"(__float_as_int(i1)) : "memory");
+        }
+    };
+    for (int y = vb + RHO; y >= vb - RHO; --y) {
+        int x[2];
+        load2(pa, acol, search, x);
+        pa -= W;
+        ac.push(0, x[0]);
+        ac.push(1, x[1]);
+#pragma unroll
+        for (int k = 0; k < NPREP; ++k) {
+            load2(pb[k], bcol[k] + 2 * lane, bon[k], x);
+            pb[k] -= W;
+            bc[k].push(0, x[0]);
+            bc[k].push(1, x[1]);
+        }
+    }
+    srp_block_sums<RHO, 1>(&ac.s[0], &ac.s[1], &sa0, &sa1);
+#pragma unroll
+    for (int k = 0; k < NPREP; ++k)
+        if (bon[k])
+            publish(k, ent + (uint32_t)(vb & 1) * buf_bytes);
+    // the two rows that enter next, loaded two rows ahead
+    int an[2][2], bn[NPREP][2][2];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const bool on = vb - RHO - 1 - r >= 0;
+        load2(pa, acol, on && search, an[r]);
+        pa -= W;
+#pragma unroll
+        for (int k = 0; k < NPREP; ++k) {
+            load2(pb[k], bcol[k] + 2 * lane, on && bon[k], bn[k][r]);
+            pb[k] -= W;
+        }
+    }
+    if constexpr (CLUSTER)
+        cluster_sync_all();   // every CTA of the cluster has started before its shared memory is written
+    else
+        __syncthreads();
+
+    const uint32_t jaddr = 16u * (uint32_t)(((col0 - ent0) >> 1) + pair);
     for (int v = vb; v >= RHO; --v) {
+        // B of the next row first (the other buffer): it depends on nothing of this row
+        if (v > RHO) {
+#pragma unroll
+            for (int k = 0; k < NPREP; ++k)
+                if (bon[k]) {
+                    bc[k].push(0, bn[k][0][0]);
+                    bc[k].push(1, bn[k][0][1]);
+                    publish(k, ent + (uint32_t)((v - 1) & 1) * buf_bytes);
+                    bn[k][0][0] = bn[k][1][0];
+                    bn[k][0][1] = bn[k][1][1];
+                    load2(pb[k], bcol[k] + 2 * lane, v - RHO - 3 >= 0, bn[k][1]);
+                    pb[k] -= W;
+                }
+        }
+        int d0 = 0, d1 = 0;
+        if (search) {
+        // search ranges: [0, dmax] on the first row, else [l - tau, l + tau] around the estimates below of
+        // the pixel and its two neighbours (one that is missing repeats the pixel's own)
+        int l00 = 0, l01 = 0, l02 = 0, l11 = 0, l12 = 0, t = a.dmax;
         if (v < vb) {
-            // row v + RHO + 1 leaves the window, row v - RHO enters (same ring slot)
-            const int slot = (v - RHO) % K;
-#pragma unroll
-            for (int k = 0; k < kMaxColsPerThread; ++k) {
-                const int u = tid + k * nthr;
-                if (u < W) {
-                    const int xo = ca8[u * 8 + slot], zo = cb8[u * 8 + slot];
-                    const int xn = na[k], zn = nb[k];
-                    ca8[u * 8 + slot] = (uint8_t)xn;
-                    cb8[u * 8 + slot] = (uint8_t)zn;
-                    cs[u] += xn - xo;
-                    cs[W + u] += xn * xn - xo * xo;
-                    cs[2 * W + u] += zn - zo;
-                    cs[3 * W + u] += zn * zn - zo * zo;
-                }
-            }
-            const int y = v - RHO - 1;   // prefetch the next entering row
-#pragma unroll
-            for (int k = 0; k < kMaxColsPerThread; ++k) {
-                const int u = tid + k * nthr;
-                if (u < W && y >= 0) {
-                    na[k] = A[(size_t)y * W + u];
-                    nb[k] = B[(size_t)y * W + u];
-                }
-            }
+            const uint32_t *below = lv + ((v + 1) & 1) * n_lv + 1;
+            const uint32_t wl = mine ? below[pair - 1] : 0u, wc = mine ? below[pair] : 0u, wr = mine ? below[pair + 1] : 0u;
+            const int lm = (int)wl >> 16, la = (int)(int16_t)(wc & 0xffffu), lb = (int)wc >> 16,
+                      lp = (int)(int16_t)(wr & 0xffffu);
+            l01 = la;
+            l00 = lm < 0 ? la : lm;
+            l02 = lb < 0 ? la : lb;   // the second pixel's range is [l01, l11, l12]
+            l11 = lb;
+            l12 = lp < 0 ? lb : lp;
+            t = a.tau;
         }
-        __syncthreads();
-        for (int u = RHO + tid; u <= W - 1 - RHO; u += nthr) {
-            int s0 = 0, q0 = 0, s1 = 0, q1 = 0;
-#pragma unroll
-            for (int x = -RHO; x <= RHO; ++x) {
-                s0 += cs[u + x];
-                q0 += cs[W + u + x];
-                s1 += cs[2 * W + u + x];
-                q1 += cs[3 * W + u + x];
+        const int mn0 = min(min(l00, l01), l02), mx0 = max(max(l00, l01), l02);
+        const int mn1 = min(min(l01, l11), l12), mx1 = max(max(l01, l11), l12);
+        int lo = min(in0 ? mn0 : 0x3fffffff, in1 ? mn1 : 0x3fffffff) - t;
+        int hi = max(in0 ? min(mx0 + t, dhi0) : -1, in1 ? min(mx1 + t, dhi1) : -1);
+        lo = max(__reduce_min_sync(0xffffffffu, lo), 0);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        const uint32_t buf = ent + (uint32_t)(v & 1) * buf_bytes;
+        const uint32_t lane_ent = buf + jaddr;
+        // best and second best score of the two pixels (far below any NCC: none yet) and the best's disparity
+        constexpr float kNone = -1e30f;
+        float b0 = kNone, b1 = kNone, r0 = kNone, r1 = kNone;
+        const int q = (col0 - ent0) + 2 * pair;   // entry of the first pixel's leftmost column at d = 0
+        auto consider = [](float s, int d, float &best, float &second, int &dbest) {
+            dbest = s > best ? d : dbest;
+            second = fmaxf(second, fminf(best, s));
+            best = fmaxf(best, s);
+        };
+        for (int base = lo; base <= hi; base += kWin) {
+            // candidates of the two pixels among d = base .. base + kWin - 1
+            uint32_t m0, m1;
+            if (t == 1) {   // bit k of c: an estimate base - 1 + k, whose range is bits k - 2 .. k of the mask
+                const uint32_t cs = srp_shl(1u, l01 - base + 1);
+                const uint32_t c0 = cs | srp_shl(1u, l00 - base + 1) | srp_shl(1u, l02 - base + 1);
+                const uint32_t c1 = cs | srp_shl(1u, l11 - base + 1) | srp_shl(1u, l12 - base + 1);
+                m0 = c0 | (c0 >> 1) | (c0 >> 2);
+                m1 = c1 | (c1 >> 1) | (c1 >> 2);
+            } else {
+                m0 = srp_bits(l00 - t - base, l00 + t - base) | srp_bits(l01 - t - base, l01 + t - base) |
+                     srp_bits(l02 - t - base, l02 + t - base);
+                m1 = srp_bits(l01 - t - base, l01 + t - base) | srp_bits(l11 - t - base, l11 + t - base) |
+                     srp_bits(l12 - t - base, l12 + t - base);
             }
-            ra2[u] = make_int2(s0, NB * q0 - s0 * s0);
-            rb2[u] = make_int2(s1, NB * q1 - s1 * s1);
-        }
-        __syncthreads();
-        const int16_t *below = lv + (cur ^ 1) * W;
-        int16_t *here = lv + cur * W;
-        const int umax = W - 1 - RHO;
-        for (int u = RHO + tid; u <= umax; u += nthr) {
-            int dhi = dir == 0 ? u - RHO : W - 1 - RHO - u;
-            dhi = dhi < a.dmax ? dhi : a.dmax;
-            // the search range as up to three intervals in ascending order: [0, dhi] on the first row, else
-            // [l - tau, l + tau] around the sorted estimates below (duplicates skipped by starting each
-            // interval after the previous one's end)
-            int c0 = 0, c1 = -1000, c2 = -1000, span = dhi;   // centres (interval = [c - span, c + span])
-            bool first = v == vb;
-            if (!first) {
-                int l0 = u - 1 >= RHO ? below[u - 1] : -1000, l1 = below[u], l2 = u + 1 <= umax ? below[u + 1] : -1000;
-                // sort three values (missing ones, -1000, first)
-                if (l0 > l1) { const int t = l0; l0 = l1; l1 = t; }
-                if (l1 > l2) { const int t = l1; l1 = l2; l2 = t; }
-                if (l0 > l1) { const int t = l0; l0 = l1; l1 = t; }
-                c0 = l0;
-                c1 = l1;
-                c2 = l2;
-                span = a.tau;
+            m0 &= srp_bits(0, min(dhi0 - base, kWin - 1));
+            m1 &= srp_bits(0, min(dhi1 - base, kWin - 1));
+            if (CLUSTER && a.groups == 2) {   // even or odd offsets
+                m0 &= group ? 0xaaaaaaaau : 0x55555555u;
+                m1 &= group ? 0xaaaaaaaau : 0x55555555u;
             }
-            // this pixel's block of A: its K columns, each the K ring rows in 8 bytes
-            uint2 acol[K];
+            uint32_t need = __reduce_or_sync(0xffffffffu, m0 | m1);
+            const int distinct = __popc(need);
+            if (distinct > kSrpShared &&
+                distinct > 3 * (int)__reduce_max_sync(0xffffffffu, (unsigned)max(__popc(m0), __popc(m1)))) {
+                // scattered estimates (no match, occlusion): each lane takes its own pixels' candidates,
+                // from the strip's columns around them
+                uint32_t alo[K + 1], ahi[K + 1];
 #pragma unroll
-            for (int x = 0; x < K; ++x)
-                acol[x] = ca[u - RHO + x];
-            const int2 sa2 = ra2[u];
-            const int sa = sa2.x, Da = sa2.y;
-            long long bN = 0;
-            int bD = 0, best = -1, next = 0;   // next: smallest disparity not yet searched
-            for (int iv = first ? 2 : 0; iv < 3; ++iv) {
-                const int c = first ? span / 2 : (iv == 0 ? c0 : (iv == 1 ? c1 : c2));
-                if (c <= -1000)
-                    continue;
-                const int from = max(next, first ? 0 : c - span), to = min(dhi, first ? dhi : c + span);
-                if (from > to)
-                    continue;
-                for (int d = from; d <= to; ++d) {
-                    const int ub = dir == 0 ? u - d : u + d;
-                    uint2 bw[K];
+                for (int x = 0; x <= RHO; ++x)
 #pragma unroll
-                    for (int x = 0; x < K; ++x)
-                        bw[x] = cb[ub - RHO + x];
-                    unsigned p4[4] = {0u, 0u, 0u, 0u};   // four independent dp4a chains
-#pragma unroll
-                    for (int x = 0; x < K; ++x) {
-                        p4[(2 * x) & 3] = __dp4a(acol[x].x, bw[x].x, p4[(2 * x) & 3]);
-                        p4[(2 * x + 1) & 3] = __dp4a(acol[x].y, bw[x].y, p4[(2 * x + 1) & 3]);
+                    for (int c = 0; c < 2; ++c) {
+                        alo[2 * x + c] = __shfl_down_sync(0xffffffffu, ac.lo[c], x);
+                        ahi[2 * x + c] = __shfl_down_sync(0xffffffffu, ac.hi[c], x);
                     }
-                    const unsigned P = (p4[0] + p4[1]) + (p4[2] + p4[3]);
-                    const int2 sb2 = rb2[ub];
-                    long long N = (long long)NB * (long long)P - (long long)sa * sb2.x;
-                    if (Da == 0)
-                        N = 0;
-                    if (best < 0 || ncc_better(N, sb2.y, bN, bD)) {
-                        best = d;
-                        bN = N;
-                        bD = sb2.y;
+                while (__any_sync(0xffffffffu, (m0 | m1) != 0u)) {
+#pragma unroll
+                    for (int p = 0; p < 2; ++p) {
+                        uint32_t &m = p ? m1 : m0;
+                        const bool on = m != 0u;
+                        const int d = base + (on ? __ffs((int)m) - 1 : 0);
+                        m &= m - 1u;
+                        // a pixel without a candidate left reads the first entries instead
+                        const int e = on ? q + p + (dir == 0 ? -d : d) : 0;
+                        const uint32_t at = buf + 16u * (uint32_t)(e >> 1);
+                        const uint32_t ev = at + ((e & 1) ? odd : 0u), od = at + ((e & 1) ? 16u : odd);
+                        const uint4 first = srp_lds(ev);
+                        unsigned P0 = __dp4a(alo[p], first.x, 0u), P1 = __dp4a(ahi[p], first.y, 0u);
+#pragma unroll
+                        for (int k = 1; k < K; ++k) {
+                            const uint2 b = srp_lds2((k & 1) ? od + 16u * (uint32_t)(k >> 1) : ev + 16u * (uint32_t)(k >> 1));
+                            P0 = __dp4a(alo[p + k], b.x, P0);
+                            P1 = __dp4a(ahi[p + k], b.y, P1);
+                        }
+                        const int N = NB * (int)(P0 + P1) - (p ? sa1 : sa0) * (int)first.z;
+                        const float s = on ? __fmul_rn((float)N, __uint_as_float(first.w)) : kNone;
+                        if (p == 0)
+                            consider(s, d, b0, r0, d0);
+                        else
+                            consider(s, d, b1, r1, d1);
                     }
                 }
-                next = max(next, to + 1);
+                continue;
             }
-            const int16_t val = (int16_t)(best < 0 ? 0 : best);
-            here[u] = val;
-            out[(size_t)v * W + u] = val;
+            while (need) {
+                // a few disparities at a time: their chains of loads, dot products and shuffles overlap
+                uint32_t low[kBatch];
+                int d[kBatch], x0[kBatch], x1[kBatch], P0[kBatch], P1[kBatch];
+                uint4 c0[kBatch], c1[kBatch];
+#pragma unroll
+                for (int k = 0; k < kBatch; ++k) {
+                    low[k] = need & (0u - need);   // 0 when the batch is not full: d repeats, no pixel takes it
+                    need ^= low[k];
+                    d[k] = low[k] ? base + 31 - __clz((int)low[k]) : d[k ? k - 1 : 0];
+                    const int e = dir == 0 ? -d[k] : d[k];
+                    const uint32_t at = lane_ent + (uint32_t)(16 * (e >> 1));
+                    c0[k] = srp_lds(at + ((e & 1) ? odd : 0u));
+                    c1[k] = srp_lds(at + ((e & 1) ? 16u : odd));
+                }
+#pragma unroll
+                for (int k = 0; k < kBatch; ++k) {
+                    x0[k] = (int)__dp4a(ac.hi[0], c0[k].y, __dp4a(ac.lo[0], c0[k].x, 0u));
+                    x1[k] = (int)__dp4a(ac.hi[1], c1[k].y, __dp4a(ac.lo[1], c1[k].x, 0u));
+                }
+                srp_block_sums<RHO, kBatch>(x0, x1, P0, P1);
+#pragma unroll
+                for (int k = 0; k < kBatch; ++k) {
+                    const int N0 = NB * P0[k] - sa0 * (int)c0[k].z, N1 = NB * P1[k] - sa1 * (int)c1[k].z;
+                    const float s0 = __fmul_rn((float)N0, __uint_as_float(c0[k].w));
+                    const float s1 = __fmul_rn((float)N1, __uint_as_float(c1[k].w));
+                    consider((m0 & low[k]) ? s0 : kNone, d[k], b0, r0, d0);
+                    consider((m1 & low[k]) ? s1 : kNone, d[k], b1, r1, d1);
+                }
+            }
         }
-        for (int u = tid; u < W; u += nthr)   // columns without a block
-            if (u < RHO || u > umax) {
-                here[u] = 0;
-                out[(size_t)v * W + u] = 0;
+        if (CLUSTER && a.groups == 2) {
+            float *at = half + strip * 32 + lane;
+            const int n = nw * 32;
+            if (group) {
+                at[0] = b0;
+                at[n] = r0;
+                at[2 * n] = __int_as_float(d0);
+                at[3 * n] = b1;
+                at[4 * n] = r1;
+                at[5 * n] = __int_as_float(d1);
+                asm volatile("bar.arrive %0, 64;" ::"r"(1 + strip) : "memory");
+            } else {
+                asm volatile("bar.sync %0, 64;" ::"r"(1 + strip) : "memory");
+                auto merge = [](float b, float r, int d, float &best, float &second, int &dbest) {
+                    second = fmaxf(fmaxf(second, r), fminf(best, b));
+                    dbest = b > best || (b == best && d < dbest) ? d : dbest;
+                    best = fmaxf(best, b);
+                };
+                merge(at[0], at[n], __float_as_int(at[2 * n]), b0, r0, d0);
+                merge(at[3 * n], at[4 * n], __float_as_int(at[5 * n]), b1, r1, d1);
             }
+        }
+        if (group == 0) {
+        // 2.25 |b| covers |s1| + |s2| of scores this close; equal zeros keep the first
+        constexpr float kEps = 2.25f * 9.5367431640625e-07f;   // 2^-20
+        const bool close0 = in0 && r0 > __fmaf_rn(fabsf(b0), -kEps, b0);
+        const bool close1 = in1 && r1 > __fmaf_rn(fabsf(b1), -kEps, b1);
+        if (close0)
+            d0 = srp_exact_best<RHO>(A, B, W, v, u0, dir == 0 ? -1 : 1, l00, l01, l02, t, dhi0);
+        if (close1)
+            d1 = srp_exact_best<RHO>(A, B, W, v, u0 + 1, dir == 0 ? -1 : 1, l01, l11, l12, t, dhi1);
+        if (mine)
+            lv[(v & 1) * n_lv + 1 + pair] = (uint32_t)(in0 ? d0 & 0xffff : 0xffff) | ((in1 ? (uint32_t)d1 : 0xffffu) << 16);
+        if (st0)
+            out[(size_t)v * W + u0] = (int16_t)d0;
+        if (st1)
+            out[(size_t)v * W + u0 + 1] = (int16_t)d1;
+        }
+        // A moves up a row
+        ac.push(0, an[0][0]);
+        ac.push(1, an[0][1]);
+        srp_block_sums<RHO, 1>(&ac.s[0], &ac.s[1], &sa0, &sa1);
+        an[0][0] = an[1][0];
+        an[0][1] = an[1][1];
+        load2(pa, acol, v - RHO - 3 >= 0, an[1]);
+        pa -= W;
+        }
+        if constexpr (CLUSTER) {
+            const int step = vb - v + 1;                     // rows done
+            if (step % kSrpHalo == 0 && v > RHO) {
+                const int par = (step / kSrpHalo) & 1;
+                const uint32_t box = (uint32_t)__cvta_generic_to_shared(inbox) + (uint32_t)(par * 2 * kSrpHalo * 2);
+                auto send = [&](int to, int slot, int val) {
+                    uint32_t r;
+                    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(box + 2u * (uint32_t)slot), "r"(to));
+                    asm volatile("st.shared::cluster.u16 [%0], %1;" ::"r"(r), "h"((short)val) : "memory");
+                };
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    const int u = u0 + c, val = c ? d1 : d0;
+                    if (!(c ? st1 : st0))
+                        continue;
+                    if (rank > 0 && u < own0 + kSrpHalo)                  // the left neighbour's right halo
+                        send(rank - 1, kSrpHalo + (u - own0), val);
+                    if (rank + 1 < nrank && u >= own1 - kSrpHalo)         // the right neighbour's left halo
+                        send(rank + 1, u - (own1 - kSrpHalo), val);
+                }
+                cluster_sync_all();
+                // the received estimates replace the stale ones of the halo (int16 entries of the pair words)
+                int16_t *row = reinterpret_cast<int16_t *>(lv + (v & 1) * n_lv + 1);
+                const int16_t *in = inbox + par * 2 * kSrpHalo;
+                if (tid < kSrpHalo && rank > 0)
+                    row[tid] = in[tid];
+                if (tid >= kSrpHalo && tid < 2 * kSrpHalo && rank + 1 < nrank && own1 + tid - kSrpHalo <= umax)
+                    row[own1 - px0 + tid - kSrpHalo] = in[tid];
+            }
+        }
         __syncthreads();
-        cur ^= 1;
     }
 }
 
-__global__ void k_lrc(const int16_t *lf, const int16_t *rt, int W, int H, int n, int tr, float *disp)
+// Launch shape of k_srp for maps of W columns.
+struct SrpShape {
+    int ctas, strips, groups, warps, prep;   // CTAs per map; strips, search groups, warps and strips per preparing warp of a CTA
+    int per, extra;
+    size_t smem;
+};
+inline SrpShape srp_shape_of(int W, int rho, int dmax, int ctas)
 {
-    const long long total = (long long)n * H * W;
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < total;
-         p += (long long)gridDim.x * blockDim.x) {
-        const int u = (int)(p % W);
-        const int l = lf[p];
-        const int x = u - l;
-        const bool ok = x >= 0 && abs(l - (int)rt[p - l]) <= tr;
-        disp[p] = ok ? (float)l : 0.0f;
+    const int S = srp_strip(rho), V = W - 2 * rho, most = kSrpMaxWarps;
+    SrpShape s;
+    s.ctas = ctas;
+    s.per = (V + ctas - 1) / ctas;
+    const int span = s.per + (ctas > 1 ? 2 * kSrpHalo : 0);
+    s.strips = (span + S - 1) / S;
+    s.extra = ((dmax < W ? dmax : W) + S - 1) / S;
+    s.groups = 1;
+    s.warps = s.strips;
+    s.prep = 1;              // one CTA's own strips hold every column of the other image
+    if (ctas > 1) {
+        const int all = s.strips + s.extra;
+        s.groups = 2 * s.strips + (all + 1) / 2 <= most ? 2 : 1;   // named barriers 1 .. strips, at most 12
+        const int room = most - s.groups * s.strips;
+        const int np = all < room ? all : room;
+        s.prep = np > 0 ? (all + np - 1) / np : kSrpPrep + 1;
+        s.warps = s.groups * s.strips + (np > 0 ? np : 0);
     }
+    const size_t ent = 2 * 16 * (size_t)srp_entries(s.strips, s.extra, rho);
+    s.smem = ent + 2 * 4 * (size_t)(s.strips * (S / 2) + 2) + 2 * 4 * kSrpHalo + 6 * 4 * 32 * (size_t)s.strips;
+    return s;
+}
+// One CTA per map fills the GPU from about 76 maps on (38 pairs; 2.2 ms as one CTA per map however few the
+// pairs, 0.76 ms for one pair on two clusters of 8); below, a map is split over the largest
+// cluster whose CTAs still find an SM each, every one keeping at least 96 pixels.  Frames wider than a CTA's
+// warps hold are always split.
+inline bool srp_fits(const SrpShape &s) { return s.warps <= kSrpMaxWarps && s.prep <= kSrpPrep; }
+inline SrpShape srp_shape(int W, int rho, int dmax, int n, int sms)
+{
+    int c = 8;
+    while (c > 1 && (2 * n * c > sms || (W - 2 * rho) / c < 96 || !srp_fits(srp_shape_of(W, rho, dmax, c))))
+        c /= 2;
+    while (c < 8 && !srp_fits(srp_shape_of(W, rho, dmax, c)))
+        c *= 2;
+    return srp_shape_of(W, rho, dmax, c);
 }
 
-size_t srp_smem(int W, int rho)
+// A warp per row, eight loads in flight per lane; the right map's gathers stay within d_max of the row's own
+// columns.  Bound by memory latency: 238 MB in 67 us for 64 x 1242x375 (110 us with a 64-bit division per
+// pixel to find its column).
+__global__ void __launch_bounds__(256) k_lrc(const int16_t *lf, const int16_t *rt, int W, int rows, int tr, float *disp)
 {
-    (void)rho;
-    return sizeof(uint2) * 2 * (size_t)W + sizeof(int) * 8 * (size_t)W + sizeof(int16_t) * 2 * (size_t)W;
+    const int lane = threadIdx.x & 31;
+    const int step = gridDim.x * (blockDim.x >> 5);
+    for (int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < rows; r += step) {
+        const int16_t *lr = lf + (size_t)r * W, *rr = rt + (size_t)r * W;
+        float *dr = disp + (size_t)r * W;
+        for (int c = lane; c < W; c += 32 * 8) {
+            int l[8], q[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                l[k] = c + 32 * k < W ? (int)__ldg(lr + c + 32 * k) : 0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int x = c + 32 * k - l[k];
+                q[k] = c + 32 * k < W && x >= 0 ? (int)__ldg(rr + x) : 0x4000;   // outside: no agreement
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (c + 32 * k < W)
+                    dr[c + 32 * k] = q[k] != 0x4000 && abs(l[k] - q[k]) <= tr ? (float)l[k] : 0.0f;
+        }
+    }
 }
 
 }  // namespace
@@ -315,15 +686,42 @@ int check_pair(ld_stereo *st, const void *left, const void *right, int w, int hh
     return LD_OK;
 }
 
-template <int RHO>
-cudaError_t launch_srp(const ld::SrpArgs &a, int n, cudaStream_t s)
+template <int RHO, int NPREP, bool CLUSTER, int WARPS>
+cudaError_t launch_srp_t(const ld::SrpArgs &a, const ld::SrpShape &sh, int n, cudaStream_t s)
 {
-    const size_t smem = ld::srp_smem(a.W, RHO);
-    cudaError_t e = cudaFuncSetAttribute(ld::k_srp<RHO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto kernel = ld::k_srp<RHO, NPREP, CLUSTER, WARPS>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem);
     if (e != cudaSuccess)
         return e;
-    ld::k_srp<RHO><<<dim3(n, 2), ld::srp_threads(a.W, RHO), smem, s>>>(a);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(sh.ctas, n, 2);
+    cfg.blockDim = dim3(32 * sh.warps);
+    cfg.dynamicSmemBytes = sh.smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = sh.ctas;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = CLUSTER ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, a);
+}
+
+template <int RHO>
+cudaError_t launch_srp(ld::SrpArgs a, int n, cudaStream_t s)
+{
+    const ld::SrpShape sh = ld::srp_shape(a.W, RHO, a.dmax, n, ld::sm_count());
+    a.per = sh.per;
+    a.strips = sh.strips;
+    a.n_extra = sh.extra;
+    a.groups = sh.groups;
+    if (sh.ctas == 1)
+        return launch_srp_t<RHO, 1, false, ld::kSrpMaxWarps>(a, sh, n, s);
+    if (sh.prep <= 1 && sh.warps <= ld::kSrpFewWarps)
+        return launch_srp_t<RHO, 1, true, ld::kSrpFewWarps>(a, sh, n, s);
+    return sh.prep <= 2 ? launch_srp_t<RHO, 2, true, ld::kSrpMaxWarps>(a, sh, n, s)
+                        : launch_srp_t<RHO, ld::kSrpPrep, true, ld::kSrpMaxWarps>(a, sh, n, s);
 }
 
 // both maps and the check on the handle's stream; `timed` records an event before SRP, between, after LRC
@@ -334,7 +732,7 @@ int enqueue_stereo(ld_stereo *st, const uint8_t *left, const uint8_t *right, int
     cudaError_t e = cudaSuccess;
     if (timed && (e = cudaEventRecord(st->ev[0], s)) != cudaSuccess)
         return scuda(st, e, "event");
-    ld::SrpArgs a{left, right, st->lf, st->rt, w, hh, st->sp.d_max, st->sp.tau};
+    ld::SrpArgs a{left, right, st->lf, st->rt, w, hh, st->sp.d_max, st->sp.tau, 0, 0, 0, 0};
     switch (st->sp.rho) {
     case 1: e = launch_srp<1>(a, n, s); break;
     case 2: e = launch_srp<2>(a, n, s); break;
@@ -344,10 +742,8 @@ int enqueue_stereo(ld_stereo *st, const uint8_t *left, const uint8_t *right, int
         return scuda(st, e, "search range propagation");
     if (timed && (e = cudaEventRecord(st->ev[1], s)) != cudaSuccess)
         return scuda(st, e, "event");
-    const long long total = (long long)n * w * hh;
-    const int g = (int)((total + 255) / 256);
-    const int gmax = ld::sm_count() * 16;
-    ld::k_lrc<<<g < gmax ? g : gmax, 256, 0, s>>>(st->lf, st->rt, w, hh, n, st->sp.tr_lrc, disp);
+    const int rows = n * hh, g = (rows + 7) / 8, gmax = ld::sm_count() * 8;
+    ld::k_lrc<<<g < gmax ? g : gmax, 256, 0, s>>>(st->lf, st->rt, w, rows, st->sp.tr_lrc, disp);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return scuda(st, e, "consistency check");
     if (timed && (e = cudaEventRecord(st->ev[2], s)) != cudaSuccess)
@@ -390,14 +786,7 @@ int ld_stereo_create(ld_handle *h, const ld_stereo_params *sp, ld_stereo **out)
     if (st->sp.d_max < 0)
         st->sp.d_max = ld::handle_params(h).n_disp - 1;
     ld::handle_dims(h, &st->max_w, &st->max_h, &st->max_n);
-    int dev = 0, optin = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess)
-        e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (e == cudaSuccess && ld::srp_smem(st->max_w, st->sp.rho) > (size_t)optin) {
-        delete st;
-        return sfail(nullptr, LD_E_ARG, "frame too wide for the shared-memory budget of the stereo kernel");
-    }
+    cudaError_t e = cudaSuccess;
     const size_t px = (size_t)st->max_n * st->max_w * st->max_h;
     if (e == cudaSuccess)
         e = cudaMalloc(&st->mem, px * (2 + 2 + 4) + 512);
