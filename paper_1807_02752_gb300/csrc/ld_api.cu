@@ -26,7 +26,6 @@ const char *const kLaunchNames[kLaunches] = {"k_vdisp", "k_road_dp", "k_fit_y", 
                                              "k_fit_x", "k_m1", "k_energy", "k_select"};
 constexpr int kGraphSlots = 4;
 constexpr int kSplitMin = 16;  // captured calls of at least this many frames run as two concurrent halves
-constexpr int kVoteCap = 12288;
 
 std::string g_create_error;
 
@@ -281,7 +280,6 @@ ld::KParams make_kparams(const ld_handle *h, int W, int H, int n)
     while ((1 << e) < half)
         ++e;
     k.e = e;
-    k.vote_cap = kVoteCap;
     const int n_ws = (2 * p.bf_rho + 1) * (2 * p.bf_rho + 1);
     for (int i = 0; i < n_ws; ++i)
         k.ws[i] = (uint16_t)h->ws_q[i];
@@ -305,7 +303,6 @@ ld::KParams make_kparams(const ld_handle *h, int W, int H, int n)
     }
     k.flat_range = flat_range(p);
     k.pmax_hint = h->w.pmax;
-    k.seg_rows = ld::vpx_seg_rows(k, (size_t)h->smem_optin - 1024);
     const bool tuned = W == h->tile_w && H == h->tile_h;
     k.tile_vdisp = tuned ? h->tile[0] : 0;
     k.tile_grad = tuned ? h->tile[1] : 0;
@@ -492,12 +489,10 @@ int enqueue_groups(ld_handle *h, const ld_group *g, int ng, bool fork)
 
 // The frames of a group list as descriptors (h->h_fdesc): each frame's own parameters and the workspace
 // seen from its slot (frames counted in the largest size, as enqueue_groups views them).  Returns the
-// launch parameters of the list's largest frame (grid and shared-memory shapes) and the V_px kernel's
-// shared memory (the largest over the frames).
+// launch parameters of the list's largest frame (grid and shared-memory shapes).
 struct MixedHalf {
     ld::KParams kl;      // launch shapes: the half's largest frame
     int first, n;        // descriptors [first, first + n)
-    size_t vpx_smem;
 };
 
 // The list is split into two halves that run concurrently: the groups by pixel count, largest first, each
@@ -535,7 +530,6 @@ int fill_descriptors(ld_handle *h, const ld_group *g, int ng, MixedHalf half[2])
     }
     int pos[2] = {0, cnt[0]};
     int Wm[2] = {16, 16}, Hm[2] = {16, 16};
-    size_t vs[2] = {0, 0};
     for (int j = 0; j < n; ++j) {
         const ld_group &gg = g[fr[j].grp];
         ld::KParams kp = make_kparams(h, gg.w, gg.h, 1);
@@ -543,7 +537,6 @@ int fill_descriptors(ld_handle *h, const ld_group *g, int ng, MixedHalf half[2])
         const int s = side[j];
         Wm[s] = std::max(Wm[s], (int)gg.w);
         Hm[s] = std::max(Hm[s], (int)gg.h);
-        vs[s] = std::max(vs[s], ld::vpx_smem_bytes(kp));
         const size_t px = (size_t)gg.w * gg.h;
         ld::FrameDesc &d = h->h_fdesc[pos[s]++];
         d.kp = kp;
@@ -557,15 +550,13 @@ int fill_descriptors(ld_handle *h, const ld_group *g, int ng, MixedHalf half[2])
         half[s].kl.tile_vdisp = half[s].kl.tile_grad = half[s].kl.tile_m1 = 0;
         half[s].first = s ? cnt[0] : 0;
         half[s].n = cnt[s];
-        half[s].vpx_smem = vs[s];
     }
     return n;
 }
 
 // The nine stages of a mixed call, one launch each over all frames (descriptors at fd, already on the
 // device), on the handle's stream.
-int enqueue_mixed_half(ld_handle *h, const ld::KParams &kl, const ld::FrameDesc *fd, int n, size_t vpx_smem,
-                       cudaStream_t s)
+int enqueue_mixed_half(ld_handle *h, const ld::KParams &kl, const ld::FrameDesc *fd, int n, cudaStream_t s)
 {
     cudaError_t e = cudaSuccess;
     for (int k = 0; k < kLaunches; ++k) {
@@ -583,7 +574,7 @@ int enqueue_mixed_half(ld_handle *h, const ld::KParams &kl, const ld::FrameDesc 
                 e = ld::launch_grad_fd(kl, fd, n, false, s);
             }
             break;
-        case 4: e = ld::launch_vpx_fd(kl, fd, n, vpx_smem, s); break;
+        case 4: e = ld::launch_vpx_fd(kl, fd, n, s); break;
         case 5: e = ld::launch_fit_x_fd(kl, fd, n, s); break;
         case 6: e = ld::launch_m1_fd(kl, fd, n, s); break;
         case 7: e = ld::launch_energy_fd(kl, fd, n, s); break;
@@ -617,7 +608,7 @@ int enqueue_mixed(ld_handle *h, const MixedHalf half[2], const ld::FrameDesc *fd
             continue;
         if ((e = cudaStreamWaitEvent(h->sub[k], h->fork, 0)) != cudaSuccess)
             return cuda_fail(h, e, "fork wait");
-        const int rc = enqueue_mixed_half(h, half[k].kl, fd + half[k].first, half[k].n, half[k].vpx_smem, h->sub[k]);
+        const int rc = enqueue_mixed_half(h, half[k].kl, fd + half[k].first, half[k].n, h->sub[k]);
         if (rc != LD_OK)
             return rc;
         if ((e = cudaEventRecord(h->join[k], h->sub[k])) != cudaSuccess ||
@@ -822,7 +813,7 @@ int ld_create(const ld_params *p, int32_t max_w, int32_t max_h, int32_t max_batc
 
     // the V_px DP needs shared memory for a block of backtrack rows and the vote bitmaps of the largest frame
     ld::KParams kmax = make_kparams(h, max_w, max_h, max_batch);
-    if (kmax.seg_rows < 1 || ld::road_smem_bytes(kmax) > (size_t)h->smem_optin - 1024) {
+    if (!ld::vpx_admits(kmax, (size_t)h->smem_optin - 1024) || ld::road_smem_bytes(kmax) > (size_t)h->smem_optin - 1024) {
         delete h;
         return fail(nullptr, LD_E_ARG, "frame too large for the shared-memory budget");
     }
@@ -910,6 +901,8 @@ int ld_create(const ld_params *p, int32_t max_w, int32_t max_h, int32_t max_batc
     }
     if (e == cudaSuccess)
         e = ld::setup_dp(h->smem_optin);
+    if (e == cudaSuccess)
+        e = ld::setup_vpx(h->smem_optin, h->p.tau_x);
     if (e == cudaSuccess)
         e = ld::setup_ransac(h->smem_optin);
     if (e == cudaSuccess)

@@ -99,9 +99,7 @@ struct KParams {
     int32_t hyps, rounds;
     uint32_t key0, key1;
     int32_t centre, e;                 // polynomial basis tau = (v - centre) / 2^e
-    int32_t seg_rows;                  // rows of DP backtrack held in shared memory by the V_px kernel
     int32_t tile_vdisp, tile_grad, tile_m1;  // rows per CTA chosen by ld_tune (0: the built-in rule)
-    int32_t vote_cap;                  // votes per frame the V_px kernel stages in shared memory
     uint16_t ws[121];                  // Eq. 16 spatial weights, Q15 (up to 32768), (2 rho + 1)^2 used
     // Taps at equal distance share one weight table in the gradient kernel.  Classes are the ranks of
     // dx^2 + dy^2 among the distinct values of the window (the kernel derives a tap's class at compile
@@ -136,7 +134,7 @@ struct Work {
     uint8_t *inl_x;      // [n][H]
     int16_t *pts;        // [n][2][3][pmax] DP path points with data (x, y, index) for the beta / gamma fits
     int32_t *npts;       // [n][2]
-    uint8_t *gbt;        // [n][max_h][vpx_row_bytes(max_w)] V_px backtrack rows below the shared-memory block
+    uint8_t *gbt;        // [n][max_h][vpx_row_bytes(max_w)] V_px backtrack rows
     int32_t *M1;         // [n][H][W]
     int32_t *xsum;       // [n][ceil(H/4)][ceil(W/4)] block sums of |G_x w_g| for the learned proposal, or null
     uint8_t *med;        // [n][H][W] median-filtered image (bilateral = 2), or null
@@ -189,9 +187,9 @@ __device__ __forceinline__ double i128_to_f64(__int128 x)
     return __dadd_rn(__dmul_rn((double)q, 4294967296.0), (double)r);
 }
 
-// Bytes of one V_px backtrack row: one byte per pair of cells (two 4-bit entries), padded to 16 bytes.
-__host__ __device__ inline int vpx_pairs(int W) { return (W + 1) >> 1; }
-__host__ __device__ inline int vpx_row_bytes(int W) { return (vpx_pairs(W) + 15) & ~15; }
+// Bytes of one V_px backtrack row: a byte per cell, lanes of at most 20 cells rounded up to four, padded to 16
+// bytes.
+__host__ __device__ inline int vpx_row_bytes(int W) { return (W + 80 + 15) & ~15; }
 
 __device__ __forceinline__ float pow2f(int k) { return __int_as_float((127 + k) << 23); }
 
@@ -264,14 +262,14 @@ cudaError_t launch_fit_y_fd(const KParams &kmax, const FrameDesc *fd, int n, cud
 cudaError_t launch_fit_x_fd(const KParams &kmax, const FrameDesc *fd, int n, cudaStream_t s);
 cudaError_t launch_grad_fd(const KParams &kmax, const FrameDesc *fd, int n, bool median_input, cudaStream_t s);
 cudaError_t launch_median_fd(const KParams &kmax, const FrameDesc *fd, int n, cudaStream_t s);
-cudaError_t launch_vpx_fd(const KParams &kmax, const FrameDesc *fd, int n, size_t smem, cudaStream_t s);
+cudaError_t launch_vpx_fd(const KParams &kmax, const FrameDesc *fd, int n, cudaStream_t s);
 cudaError_t launch_m1_fd(const KParams &kmax, const FrameDesc *fd, int n, cudaStream_t s);
 cudaError_t launch_energy_fd(const KParams &kmax, const FrameDesc *fd, int n, cudaStream_t s);
 cudaError_t launch_select_fd(const KParams &kmax, const FrameDesc *fd, int n, cudaStream_t s);
 size_t road_smem_bytes(const KParams &kp);
-size_t vpx_smem_bytes(const KParams &kp);
-int vpx_seg_rows(const KParams &kp, size_t budget);
+bool vpx_admits(const KParams &kp, size_t budget);
 cudaError_t setup_dp(int smem_optin);
+cudaError_t setup_vpx(int smem_optin, int tau);
 cudaError_t setup_ransac(int smem_optin);
 cudaError_t setup_grad(int smem_optin);
 cudaError_t setup_lpv(int smem_optin);
