@@ -21,10 +21,23 @@
 //     Eq. 20 - and solved in float64 by Gaussian elimination with partial pivoting; a pivot below 2^-40 is
 //     singular).
 //
-// GB300 mapping: every THREAD fits one hypothesis in float32 (GB300's FP64 pipe is narrow, so float64 is
-// kept to the final solve); inlier counts put consecutive hypotheses on consecutive lanes against the same
-// point (broadcast loads, independent iterations); the final fit reduces each exact int128 sum on its own
-// warp and solves the normal equations on one warp, one column per lane.
+// GB300 mapping (one CTA per frame; the stages are chains of latencies):
+//   - the working set stays compacted in shared memory in point order, as (x, y) pairs for the draws and the
+//     exact sums and as (tau, -y) floats for the inlier test, so a draw is one load and a test one more;
+//   - every THREAD fits one hypothesis in float32 (GB300's FP64 pipe is narrow, so float64 is kept to the final
+//     solve), the four draws of a Philox block loaded together.  The threads of a hypothesis (four with 64
+//     hypotheses) fit it redundantly, which costs less than handing the coefficients over, and share the
+//     points of its inlier count, two points per packed float instruction;
+//   - every warp finds the round's winner for itself (one max-reduction of count and index), and the working
+//     set is compacted with ballots: three barriers a round;
+//   - the final sums are formed in 64-bit integers (powers from t^6 on as two halves), reduced over a warp in
+//     27-bit limbs by integer reductions; the normal equations are solved on one warp, one column per lane,
+//     with one division per elimination step (each lane one factor).
+// Measured (GB300), against serial draws with dependent loads, int128 sums and shuffles: k_fit<5> 78 -> 47 us
+// and k_fit<3> 27 -> 18 us on 64 x 1242x375, 45 -> 31 and 22 -> 16 us on one such frame.  A round of 64
+// hypotheses over 250 points is about 6000 cycles (fitting 2200, counting 2700, the rest barriers and
+// compaction); the float64 solve of the quartic is 12 500 cycles (a double addition takes 63 cycles here, a
+// division 560) and bounds what is left.
 #include "ld_internal.cuh"
 
 namespace ld {
@@ -35,6 +48,8 @@ constexpr int kFitThreads = 256;
 constexpr int kNW = kFitThreads / 32;
 
 __device__ __forceinline__ double p2d(int k) { return __longlong_as_double((long long)(1023 + k) << 52); }
+
+__device__ __forceinline__ long long magnitude(double x) { return __double_as_longlong(x) & 0x7fffffffffffffffll; }
 
 // Normal equations of M unknowns from exact sums S = (Sx[0 .. 2M-2], Sy[0 .. M-1]), Sx[k] = sum t^k,
 // Sy[k] = sum y t^k: A[r][c] = Sx[r + c] 2^-(r+c)e, b[r] = Sy[r] 2^-re (exact power-of-two column scaling),
@@ -60,15 +75,17 @@ __device__ int solve_normal_warp(const __int128 *S, int e, double *coef)
 #pragma unroll
         for (int i = 0; i < M; ++i)
             pc[i] = __shfl_sync(0xffffffffu, col[i], k);
+        // magnitudes compared as integers (finite values order like their bits; a double comparison takes as
+        // long as a double addition, 63 cycles)
         int piv = k;
-        double pa = fabs(pc[k]);
+        long long pa = magnitude(pc[k]);
 #pragma unroll
         for (int i = k + 1; i < M; ++i)
-            if (fabs(pc[i]) > pa) {
-                pa = fabs(pc[i]);
+            if (magnitude(pc[i]) > pa) {
+                pa = magnitude(pc[i]);
                 piv = i;
             }
-        if (!(pa >= 0x1p-40))
+        if (pa < magnitude(0x1p-40))
             return -1;
 #pragma unroll
         for (int i = k + 1; i < M; ++i)
@@ -80,11 +97,18 @@ __device__ int solve_normal_warp(const __int128 *S, int e, double *coef)
                 pc[k] = pc[i];
                 pc[i] = t;
             }
-        if (c > k) {
+        if (k + 1 < M) {
+            // lane i divides for row i; the factors are then handed round
+            double num = pc[M - 1];
+#pragma unroll
+            for (int i = k + 1; i < M - 1; ++i)
+                num = lane == i ? pc[i] : num;
+            const double fct = __ddiv_rn(num, pc[k]);
 #pragma unroll
             for (int i = k + 1; i < M; ++i) {
-                const double fct = __ddiv_rn(pc[i], pc[k]);
-                col[i] = __dsub_rn(col[i], __dmul_rn(fct, col[k]));
+                const double fi = __shfl_sync(0xffffffffu, fct, i);
+                if (c > k)
+                    col[i] = __dsub_rn(col[i], __dmul_rn(fi, col[k]));
             }
         }
     }
@@ -106,48 +130,14 @@ __device__ int solve_normal_warp(const __int128 *S, int e, double *coef)
     return 0;
 }
 
-__device__ __forceinline__ __int128 shfl_down_i128(__int128 v, int d)
+// Sum over the warp of a signed 64-bit integer (whose true sum fits 64 bits), on every lane.
+__device__ __forceinline__ long long warp_sum64(long long v)
 {
-    long long lo = (long long)(unsigned long long)v;
-    long long hi = (long long)(v >> 64);
-    lo = __shfl_down_sync(0xffffffffu, lo, d);
-    hi = __shfl_down_sync(0xffffffffu, hi, d);
-    return ((__int128)hi << 64) | (__int128)(unsigned long long)lo;
-}
-
-// Ascending list of the indices j < n with flag[j] != 0; returns the count.  chunk: >= n/32 + 2 ints.
-__device__ int block_compact(const uint8_t *flag, int n, int16_t *list, int *chunk)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nch = (n + 31) >> 5;
-    for (int c = warp; c < nch; c += kNW) {
-        const int j = (c << 5) + lane;
-        const unsigned m = __ballot_sync(0xffffffffu, j < n && flag[j]);
-        if (lane == 0)
-            chunk[c] = __popc(m);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int s = 0;
-        for (int c = 0; c < nch; ++c) {
-            const int t = chunk[c];
-            chunk[c] = s;
-            s += t;
-        }
-        chunk[nch] = s;
-    }
-    __syncthreads();
-    for (int c = warp; c < nch; c += kNW) {
-        const int j = (c << 5) + lane;
-        const bool b = j < n && flag[j];
-        const unsigned m = __ballot_sync(0xffffffffu, b);
-        if (b)
-            list[chunk[c] + __popc(m & ((1u << lane) - 1u))] = (int16_t)j;
-    }
-    __syncthreads();
-    const int cnt = chunk[nch];
-    __syncthreads();
-    return cnt;
+    constexpr unsigned kAll = 0xffffffffu, kLimb = (1u << 27) - 1u;   // 32 limbs of 27 bits fit 32 bits
+    const unsigned l0 = __reduce_add_sync(kAll, (unsigned)v & kLimb);
+    const unsigned l1 = __reduce_add_sync(kAll, (unsigned)(v >> 27) & kLimb);
+    const int l2 = __reduce_add_sync(kAll, (int)(v >> 54));
+    return (long long)((unsigned long long)l0 + ((unsigned long long)l1 << 27) + ((unsigned long long)(long long)l2 << 54));
 }
 
 template <typename T>
@@ -159,103 +149,174 @@ __device__ __forceinline__ T *carve(unsigned char *&p, size_t count)
     return r;
 }
 
-// One hypothesis: the minimal sample of Philox draws and the polynomial through it in Newton form
-// (nodes = the sample's tau in draw order, c = float32 divided differences, computed in place).
+// One hypothesis: the minimal sample of Philox draws from the ns points xy (x << 16 | y) and the polynomial
+// through it in Newton form (nodes = the sample's tau in draw order, c = float32 divided differences).
 template <int M>
-__device__ bool hypothesis(const KParams &kp, const int16_t *xs, const int16_t *ys, const int16_t *list, int ns,
-                           int stage, int round, int h, float *c, float *nodes)
+__device__ __forceinline__ bool hypothesis(const KParams &kp, const uint32_t *xy, const float *rcp, int ns, int stage, int round,
+                                           int h, float sc, float *c, float *nodes)
 {
-    int pick[M];
+    int X[M], Y[M];
+#pragma unroll
+    for (int k = 0; k < M; ++k)
+        X[k] = -1, Y[k] = 0;   // no point has x = -1
     int got = 0;
-    uint4 blk = make_uint4(0u, 0u, 0u, 0u);
-    for (int j = 0; j < 8 * M && got < M; ++j) {
-        if ((j & 3) == 0)
-            blk = philox4x32_10(make_uint4(((uint32_t)stage << 24) | (uint32_t)round, (uint32_t)h, (uint32_t)(j >> 2), 0u),
-                                kp.key0, kp.key1);
-        const uint32_t wv = (j & 3) == 0 ? blk.x : (j & 3) == 1 ? blk.y : (j & 3) == 2 ? blk.z : blk.w;
-        const int idx = (int)(((unsigned long long)wv * (unsigned long long)ns) >> 32);
-        if (!LD_IN(idx, ns, CK_FIT_SAMPLE))
-            continue;
-        const int pt = list[idx];
-        bool dup = false;
-        for (int q = 0; q < got; ++q)
-            dup |= (pick[q] == pt) | (xs[pick[q]] == xs[pt]);
-        if (!dup)
-            pick[got++] = pt;
+#pragma unroll 1
+    for (int b = 0; b < 2 * M && got < M; ++b) {
+        const uint4 w = philox4x32_10(make_uint4(((uint32_t)stage << 24) | (uint32_t)round, (uint32_t)h, (uint32_t)b, 0u),
+                                      kp.key0, kp.key1);
+        const uint32_t wv[4] = {w.x, w.y, w.z, w.w};
+        uint32_t p[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int idx = (int)__umulhi(wv[q], (uint32_t)ns);
+            p[q] = LD_IN(idx, ns, CK_FIT_SAMPLE) ? xy[idx] : 0u;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int x = (int)(p[q] >> 16);
+            bool take = got < M;   // a point or a row drawn before is skipped
+#pragma unroll
+            for (int k = 0; k < M; ++k)
+                take = take && X[k] != x;
+#pragma unroll
+            for (int k = 0; k < M; ++k)
+                if (take && k == got) {
+                    X[k] = x;
+                    Y[k] = (int)(p[q] & 0xffffu);
+                }
+            got += take ? 1 : 0;
+        }
     }
     if (got < M)
         return false;
-    const float sc = pow2f(-kp.e);
 #pragma unroll
     for (int q = 0; q < M; ++q) {
-        nodes[q] = __fmul_rn((float)(xs[pick[q]] - kp.centre), sc);
-        c[q] = (float)ys[pick[q]];
+        nodes[q] = __fmul_rn((float)(X[q] - kp.centre), sc);
+        c[q] = (float)Y[q];
     }
+    // Divided differences.  A divisor is (x_i - x_j) 2^-e, whose reciprocal the table holds correctly rounded,
+    // so the quotient takes a product and two remainder corrections (P. Markstein, IBM J. Res. Dev. 34, 1990:
+    // from a faithful quotient and the correctly rounded reciprocal, the corrected quotient is the correctly
+    // rounded one), without the branch of the general division.  Its remainders are exact unless the dividend
+    // is tiny: then the sample is divided in the general way.
+    float d[M];
+    bool tiny = false;
+#pragma unroll
+    for (int i = 0; i < M; ++i)
+        d[i] = c[i];
 #pragma unroll
     for (int k = 1; k < M; ++k)
 #pragma unroll
-        for (int i = M - 1; i >= k; --i)
-            c[i] = __fdiv_rn(__fsub_rn(c[i], c[i - 1]), __fsub_rn(nodes[i], nodes[i - k]));
+        for (int i = M - 1; i >= k; --i) {
+            const int dx = X[i] - X[i - k];
+            const float r = rcp[abs(dx)], y = dx < 0 ? -r : r;
+            const float num = __fsub_rn(d[i], d[i - 1]), den = __fsub_rn(nodes[i], nodes[i - k]);
+            tiny = tiny || (num != 0.0f && fabsf(num) < 0x1p-60f);
+            float q = __fmul_rn(num, y);
+            q = __fmaf_rn(__fmaf_rn(-q, den, num), y, q);
+            d[i] = __fmaf_rn(__fmaf_rn(-q, den, num), y, q);
+        }
+    if (tiny) {
+#pragma unroll
+        for (int k = 1; k < M; ++k)
+#pragma unroll
+            for (int i = M - 1; i >= k; --i)
+                c[i] = __fdiv_rn(__fsub_rn(c[i], c[i - 1]), __fsub_rn(nodes[i], nodes[i - k]));
+    } else {
+#pragma unroll
+        for (int i = 0; i < M; ++i)
+            c[i] = d[i];
+    }
     return true;
 }
 
-// Inlier test of a Newton-form hypothesis: (y - p(tau))^2 < tr, nested evaluation in float32.
+// Inlier test of a Newton-form hypothesis: (y - p(tau))^2 < tr, nested evaluation in float32 (one rounding per
+// operation), for ty = (tau, -y); nn: the negated nodes.
 template <int M>
-__device__ __forceinline__ bool newton_inlier(const float *c, const float *nodes, int x, int y, int centre, float sc,
-                                              float tr)
+__device__ __forceinline__ bool newton_inlier(const float *c, const float *nn, float2 ty, float tr)
 {
-    const float tau = __fmul_rn((float)(x - centre), sc);
     float p = c[M - 1];
 #pragma unroll
     for (int k = M - 2; k >= 0; --k)
-        p = __fadd_rn(__fmul_rn(p, __fsub_rn(tau, nodes[k])), c[k]);
-    const float r = __fsub_rn((float)y, p);
+        p = __fadd_rn(__fmul_rn(p, __fadd_rn(ty.x, nn[k])), c[k]);
+    const float r = __fadd_rn(p, ty.y);   // p - y: its square is that of y - p
     return __fmul_rn(r, r) < tr;
+}
+// Packed product, each half rounded once: a fused multiply-add of minus zero, computed so that the compiler does
+// not know its value (a packed multiplication is contracted with a packed addition that follows it, whatever
+// the contraction flags say, and a known zero turns the multiply-add back into that multiplication).
+__device__ __forceinline__ float2 mul2(float2 a, float2 b, float2 minus_zero) { return __ffma2_rn(a, b, minus_zero); }
+
+// The inlier test of two points at once (packed float: each half rounded as the scalar operation).
+template <int M>
+__device__ __forceinline__ int newton_inlier2(const float *c, const float *nn, float2 a, float2 b, float tr, float2 mz)
+{
+    const float2 tau = make_float2(a.x, b.x);
+    float2 p = make_float2(c[M - 1], c[M - 1]);
+#pragma unroll
+    for (int k = M - 2; k >= 0; --k)
+        p = __fadd2_rn(mul2(p, __fadd2_rn(tau, make_float2(nn[k], nn[k])), mz), make_float2(c[k], c[k]));
+    const float2 r = __fadd2_rn(p, make_float2(a.y, b.y));
+    const float2 s = mul2(r, r, mz);
+    return (s.x < tr ? 1 : 0) + (s.y < tr ? 1 : 0);
 }
 
 template <int M>
 __device__ __forceinline__ void fit_body(const KParams &kp, const Work &w, const int f)
 {
     constexpr int stage = M == 3 ? 0 : 1;
+    constexpr int kPer = (LD_MAX_H + kFitThreads - 1) / kFitThreads;   // points a thread compacts (D <= LD_MAX_H)
+    constexpr int NS = 3 * M - 1;   // exact sums: t^k, k <= 2M - 2, then y t^k, k < M
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ double coef_s[M];
     __shared__ int sh[4];
     const int H = kp.H, P = w.pmax;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const FrameState fs0 = w.fs[f];
-    if (stage == 1 && (fs0.flags & LD_F_NO_LANES))
-        return;
     const int n0 = w.npts[f * 2 + stage];
-    const int n = LD_IN(n0, P + 1, CK_FIT_NPTS) ? n0 : 0;   // a point list holds at most P points
     const int16_t *gp = w.pts + ((size_t)f * 2 + stage) * 3 * P;
 
     unsigned char *p = smem;
-    int16_t *xs = carve<int16_t>(p, P);
-    int16_t *ys = carve<int16_t>(p, P);
+    uint32_t *xy = carve<uint32_t>(p, P);
+    float2 *ty = carve<float2>(p, P);
     int16_t *pid = carve<int16_t>(p, P);
-    uint8_t *member = carve<uint8_t>(p, P);
-    int16_t *list = carve<int16_t>(p, P);
-    int *chunk = carve<int>(p, (P + 31) / 32 + 2);
-    int *hyp_ok = carve<int>(p, kMaxHyps);
-    int *hyp_cnt = carve<int>(p, kMaxHyps);
-    float *hyp_cf = carve<float>(p, kMaxHyps * 2 * M);  // per hypothesis: M divided differences, M nodes
-    __int128 *red = carve<__int128>(p, kNW * (3 * M - 1));
+    int *chunk = carve<int>(p, kPer * kNW);
+    int *count = carve<int>(p, kMaxHyps);               // inliers of each hypothesis; negative: void
+    float *rcp = carve<float>(p, H);                    // 2^e / i, correctly rounded
+    float *hyp_cf = carve<float>(p, kMaxHyps * 2 * M);  // per hypothesis: M divided differences, M negated nodes
+    __int128 *red = carve<__int128>(p, NS);
+    long long *red64 = carve<long long>(p, kNW * (NS + 3));
     int *redc = carve<int>(p, kNW);
-
-    for (int j = tid; j < n; j += kFitThreads) {
-        xs[j] = gp[j];
-        ys[j] = gp[P + j];
-        pid[j] = gp[2 * P + j];
-        member[j] = 1;
-    }
-    __syncthreads();
 
     const int centre = kp.centre;
     const float sc = pow2f(-kp.e);
     const float tr = stage == 0 ? kp.tr_y : kp.tr_x;
-    int fl = 0, round = 0;
+    const int n = LD_IN(n0, P + 1, CK_FIT_NPTS) ? n0 : 0;
+    for (int i = tid; i < H; i += kFitThreads)
+        rcp[i] = __fmul_rn(__frcp_rn((float)max(i, 1)), pow2f(kp.e));
+    for (int i = tid; i < kp.hyps; i += kFitThreads)
+        count[i] = 0;
+    const int most = min(P, stage == 0 ? kp.D : H);         // points there can be (the list's memory holds P)
+#pragma unroll 2
+    for (int j = tid; j < most; j += kFitThreads) {
+        const int x = gp[j], y = gp[P + j];
+        xy[j] = (uint32_t)(x & 0xffff) << 16 | (uint32_t)(y & 0xffff);
+        ty[j] = make_float2(__fmul_rn((float)(x - centre), sc), -(float)y);
+        pid[j] = gp[2 * P + j];
+    }
+    if (stage == 1 && (fs0.flags & LD_F_NO_LANES))
+        return;
+    const int n_inl = stage == 0 ? kp.D : H;
+    uint8_t *inl = stage == 0 ? w.inl_y + (size_t)f * n_inl : w.inl_x + (size_t)f * n_inl;
+    for (int i = tid; i < n_inl; i += kFitThreads)
+        inl[i] = 0;
+    __syncthreads();
+
+    // hypothesis h is fitted and counted by `groups` threads, h + g nh
+    const int nh = kp.hyps, groups = min(kFitThreads / nh, 32), h = tid % nh, g = tid / nh;
+    const float2 mz = make_float2(__fmul_rn(sc, -0.0f), __fmul_rn(sc, -0.0f));   // -0 (see mul2)
+    int fl = 0, round = 0, ns = n;
     for (;;) {
-        const int ns = block_compact(member, n, list, chunk);
         if (ns < M) {
             fl |= 2;
             break;
@@ -264,191 +325,173 @@ __device__ __forceinline__ void fit_body(const KParams &kp, const Work &w, const
             fl |= 1;
             break;
         }
-        for (int h = tid; h < kp.hyps; h += kFitThreads) {
-            float c[M], nodes[M];
-            const bool ok = hypothesis<M>(kp, xs, ys, list, ns, stage, round, h, c, nodes);
-            hyp_ok[h] = ok;
+        if (g < groups) {
+            float c[M], nn[M];
+            const bool ok = hypothesis<M>(kp, xy, rcp, ns, stage, round, h, sc, c, nn);
+            int cnt = -1;
+            if (ok) {
+                cnt = 0;
 #pragma unroll
-            for (int k = 0; k < M; ++k) {
-                hyp_cf[h * 2 * M + k] = ok ? c[k] : 0.0f;
-                hyp_cf[h * 2 * M + M + k] = ok ? nodes[k] : 0.0f;
-            }
-        }
-        __syncthreads();
-        // inlier counts: consecutive lanes take consecutive hypotheses against the same point (broadcast
-        // point loads, independent iterations); a thread adds its count when its hypothesis changes
-        for (int h = tid; h < kp.hyps; h += kFitThreads)
-            hyp_cnt[h] = hyp_ok[h] ? 0 : -1;
-        __syncthreads();
-        {
-            const int nh = kp.hyps, dh = kFitThreads % nh, dq = kFitThreads / nh;
-            if (dh == 0) {
-                // the thread's hypothesis is fixed: a plain strided loop the compiler can overlap
-                const int h = tid % nh;
-                if (hyp_ok[h]) {
-                    float cf[2 * M];
-#pragma unroll
-                    for (int k = 0; k < 2 * M; ++k)
-                        cf[k] = hyp_cf[h * 2 * M + k];
-                    int c = 0;
+                for (int k = 0; k < M; ++k)
+                    nn[k] = -nn[k];
+                int q = g;
 #pragma unroll 4
-                    for (int q = tid / nh; q < ns; q += dq) {
-                        const int j = list[q];
-                        c += newton_inlier<M>(cf, cf + M, xs[j], ys[j], centre, sc, tr);
-                    }
-                    if (c)
-                        atomicAdd(&hyp_cnt[h], c);
-                }
-            } else {
-                int h = tid % nh, q = tid / nh, cur = -1, c = 0;
-                bool ok = false;
-                float cf[2 * M];
-                for (; q < ns; q += dq) {
-                    if (h != cur) {
-                        if (ok && c)
-                            atomicAdd(&hyp_cnt[cur], c);
-                        cur = h;
-                        c = 0;
-                        ok = hyp_ok[h] != 0;
+                for (; q + groups < ns; q += 2 * groups)
+                    cnt += newton_inlier2<M>(c, nn, ty[q], ty[q + groups], tr, mz);
+                if (q < ns)
+                    cnt += newton_inlier<M>(c, nn, ty[q], tr) ? 1 : 0;
+                if (g == 0)
 #pragma unroll
-                        for (int k = 0; k < 2 * M; ++k)
-                            cf[k] = hyp_cf[h * 2 * M + k];
+                    for (int k = 0; k < M; ++k) {
+                        hyp_cf[h * 2 * M + k] = c[k];
+                        hyp_cf[h * 2 * M + M + k] = nn[k];
                     }
-                    if (ok) {
-                        const int j = list[q];
-                        c += newton_inlier<M>(cf, cf + M, xs[j], ys[j], centre, sc, tr);
-                    }
-                    h += dh;
-                    if (h >= nh) {
-                        h -= nh;
-                        ++q;
-                    }
-                }
-                if (ok && c)
-                    atomicAdd(&hyp_cnt[cur], c);
             }
+            if (cnt > 0 || (cnt < 0 && g == 0))
+                atomicAdd(&count[h], cnt > 0 ? cnt : -(1 << 20));
         }
         __syncthreads();
-        if (warp == 0) {
-            int bc = -1, bh = 0x7fffffff;
-            for (int h = lane; h < kp.hyps; h += 32)
-                if (hyp_cnt[h] > bc) {
-                    bc = hyp_cnt[h];
-                    bh = h;
-                }
-            for (int d = 16; d > 0; d >>= 1) {
-                const int oc = __shfl_down_sync(0xffffffffu, bc, d);
-                const int oh = __shfl_down_sync(0xffffffffu, bh, d);
-                if (oc > bc || (oc == bc && oh < bh)) {
-                    bc = oc;
-                    bh = oh;
-                }
-            }
-            if (lane == 0) {
-                sh[0] = bh;
-                sh[1] = bc;
-            }
-        }
-        __syncthreads();
-        const int bh = sh[0], bc = sh[1];
+        // the winner: most inliers, then the lowest index (count << 8 | 255 - index; negative when none is valid)
+        int best = -1;
+        for (int i = lane; i < nh; i += 32)
+            best = max(best, count[i] * 256 + (255 - i));
+        best = __reduce_max_sync(0xffffffffu, best);
         ++round;
-        if (bc < 0) {
+        if (best < 0) {
             fl |= 2;
             break;
         }
+        const int bh = 255 - (best & 255), bc = best >> 8;
         float cf[2 * M];
 #pragma unroll
         for (int k = 0; k < 2 * M; ++k)
             cf[k] = hyp_cf[bh * 2 * M + k];
-        for (int j = tid; j < n; j += kFitThreads)
-            if (member[j] && !newton_inlier<M>(cf, cf + M, xs[j], ys[j], centre, sc, tr))
-                member[j] = 0;
+        // the winner's inliers stay, in order: each warp flags its chunks of 32 points, then places them
+        uint32_t kxy[kPer];
+        float2 kty[kPer];
+        int16_t kid[kPer];
+        unsigned keep[kPer];
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            const int j = tid + i * kFitThreads;
+            keep[i] = 0u;
+            if (i * kFitThreads >= ns)
+                break;
+            if (j < ns) {
+                kxy[i] = xy[j];
+                kty[i] = ty[j];
+                kid[i] = pid[j];
+            }
+            keep[i] = __ballot_sync(0xffffffffu, j < ns && newton_inlier<M>(cf, cf + M, kty[i], tr));
+            if (lane == 0)
+                chunk[i * kNW + warp] = __popc(keep[i]);
+        }
         __syncthreads();
-        if ((long long)kp.eps_den * bc >= (long long)kp.eps_num * ns)
+        for (int i = tid; i < nh; i += kFitThreads)
+            count[i] = 0;
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            if (i * kFitThreads >= ns)
+                break;
+            const int me = i * kNW + warp;   // chunks before this one
+            int before = lane < me ? chunk[lane] : 0;
+            if (kPer * kNW > 32 && lane + 32 < me)
+                before += chunk[lane + 32];
+            before = __reduce_add_sync(0xffffffffu, before);
+            if (keep[i] >> lane & 1u) {
+                const int at = before + __popc(keep[i] & ((1u << lane) - 1u));
+                xy[at] = kxy[i];
+                ty[at] = kty[i];
+                pid[at] = kid[i];
+            }
+        }
+        const bool done = (long long)kp.eps_den * bc >= (long long)kp.eps_num * ns;
+        ns = bc;
+        __syncthreads();
+        if (done)
             break;
     }
-    // final least squares over the remaining set: exact sums (sum t^k for k <= 2M-2, then
-    // sum y t^k for k < M), then the normal equations solved on one warp
+    for (int j = tid; j < ns; j += kFitThreads)   // final membership (cleared before the rounds)
+        if (LD_IN(pid[j], n_inl, CK_FIT_ROW))
+            inl[pid[j]] = 1;
+    // final least squares over the remaining set: exact sums (sum t^k for k <= 2M-2, then sum y t^k for k < M),
+    // then the normal equations solved on one warp.  |t| < 2^10, y < 2^13 and at most 2^11 points: sums of t^k
+    // up to k = 5 and of y t^k up to k = 4 fit 64 bits; t^6 .. t^8 are summed as 2^32 hi + lo.
     if (!(fl & 2)) {
-        constexpr int NS = 3 * M - 1;
-        if constexpr (M == 5) {
-            // each thread's points: the powers of t built once per point, all NS sums at a time
-            __int128 acc[NS];
+        constexpr int N64 = 2 * M - 1 > 6 ? 6 : 2 * M - 1;   // powers 0 .. N64 - 1 in 64 bits
+        constexpr int NHI = 2 * M - 1 - N64;
+        long long sx[N64], sy[M], hi[NHI > 0 ? NHI : 1], lo[NHI > 0 ? NHI : 1];
 #pragma unroll
-            for (int k = 0; k < NS; ++k)
-                acc[k] = 0;
-            int cnt = 0;
-            for (int j = tid; j < n; j += kFitThreads)
-                if (member[j]) {
-                    const __int128 t = (__int128)(xs[j] - centre), y = (__int128)ys[j];
-                    __int128 pw = 1;
+        for (int k = 0; k < N64; ++k)
+            sx[k] = 0;
 #pragma unroll
-                    for (int k = 0; k < 2 * M - 1; ++k) {
-                        acc[k] += pw;
-                        if (k < M)
-                            acc[2 * M - 1 + k] += y * pw;
-                        pw *= t;
-                    }
-                    ++cnt;
-                }
-            // warp sums, then the warps' partial sums added by one warp (integer: the order does not matter)
+        for (int k = 0; k < M; ++k)
+            sy[k] = 0;
 #pragma unroll
-            for (int k = 0; k < NS; ++k)
+        for (int k = 0; k < NHI; ++k)
+            hi[k] = lo[k] = 0;
+        for (int j = tid; j < ns; j += kFitThreads) {
+            const uint32_t v = xy[j];
+            const long long t = (int)(v >> 16) - centre, y = (int)(v & 0xffffu);
+            long long pw = 1;
 #pragma unroll
-                for (int d = 16; d > 0; d >>= 1)
-                    acc[k] += shfl_down_i128(acc[k], d);
-            cnt = __reduce_add_sync(0xffffffffu, cnt);
-            if (lane == 0) {
-#pragma unroll
-                for (int k = 0; k < NS; ++k)
-                    red[warp * NS + k] = acc[k];
-                redc[warp] = cnt;
+            for (int k = 0; k < N64; ++k) {
+                sx[k] += pw;
+                if (k < M)
+                    sy[k] += y * pw;
+                if (k + 1 < N64)
+                    pw *= t;
             }
-            __syncthreads();
-            if (warp == 0) {
-                __int128 s = 0;
-                int c = 0;
-                if (lane < NS)
-                    for (int wv = 0; wv < kNW; ++wv)
-                        s += red[wv * NS + lane];
-                for (int wv = 0; wv < kNW; ++wv)
-                    c += redc[wv];
-                __syncwarp();
-                if (lane < NS)
-                    red[lane] = s;
-                if (lane == 0)
-                    redc[0] = c;
-            }
-            __syncthreads();
-        } else {   // M = 3: one warp per sum measured faster (8 sums: one round of the 8 warps)
-            for (int sidx = warp; sidx < NS; sidx += kNW) {
-                const int pk = sidx < 2 * M - 1 ? sidx : sidx - (2 * M - 1);
-                __int128 acc = 0;
-                int cnt = 0;
-                for (int j = lane; j < n; j += 32)
-                    if (member[j]) {
-                        const __int128 t = (__int128)(xs[j] - centre);
-                        __int128 pw = sidx < 2 * M - 1 ? (__int128)1 : (__int128)ys[j];
-                        for (int k = 0; k < pk; ++k)
-                            pw *= t;
-                        acc += pw;
-                        ++cnt;
-                    }
+            long long q = t;   // t^5 t^(k+1)
 #pragma unroll
-                for (int d = 16; d > 0; d >>= 1)
-                    acc += shfl_down_i128(acc, d);
-                cnt = __reduce_add_sync(0xffffffffu, cnt);
-                if (lane == 0) {
-                    red[sidx] = acc;
-                    if (sidx == 0)
-                        redc[0] = cnt;
-                }
+            for (int k = 0; k < NHI; ++k) {
+                const unsigned long long l = (unsigned long long)pw * (unsigned long long)q;
+                const long long hh = __mul64hi(pw, q);
+                hi[k] += (long long)((unsigned long long)hh << 32 | l >> 32);
+                lo[k] += (long long)(l & 0xffffffffull);
+                q *= t;
             }
-            __syncthreads();
         }
+#pragma unroll
+        for (int k = 0; k < N64; ++k)
+            sx[k] = warp_sum64(sx[k]);
+#pragma unroll
+        for (int k = 0; k < M; ++k)
+            sy[k] = warp_sum64(sy[k]);
+#pragma unroll
+        for (int k = 0; k < NHI; ++k) {
+            hi[k] = warp_sum64(hi[k]);
+            lo[k] = warp_sum64(lo[k]);
+        }
+        if (lane == 0) {
+            long long *r = red64 + warp * (NS + 3);
+#pragma unroll
+            for (int k = 0; k < N64; ++k)
+                r[k] = sx[k];
+#pragma unroll
+            for (int k = 0; k < NHI; ++k) {
+                r[N64 + k] = hi[k];
+                r[NS + k] = lo[k];
+            }
+#pragma unroll
+            for (int k = 0; k < M; ++k)
+                r[2 * M - 1 + k] = sy[k];
+        }
+        __syncthreads();
         if (warp == 0) {
+            if (lane < NS) {
+                long long a = 0, b = 0;
+                const bool two = lane >= N64 && lane < 2 * M - 1;
+                for (int wv = 0; wv < kNW; ++wv) {
+                    a += red64[wv * (NS + 3) + lane];
+                    if (two)
+                        b += red64[wv * (NS + 3) + NS + lane - N64];
+                }
+                red[lane] = two ? ((__int128)a << 32) + b : (__int128)a;
+            }
+            __syncwarp();
             double cd[M];
-            int ok = redc[0] >= M ? solve_normal_warp<M>(red, kp.e, cd) == 0 : 0;
+            int ok = ns >= M ? solve_normal_warp<M>(red, kp.e, cd) == 0 : 0;
             if (lane == 0) {
                 if (ok)
                     for (int k = 0; k < M; ++k)
@@ -463,13 +506,6 @@ __device__ __forceinline__ void fit_body(const KParams &kp, const Work &w, const
 
     const double sc64 = p2d(-kp.e);
     if (stage == 0) {
-        uint8_t *inl = w.inl_y + (size_t)f * kp.D;
-        for (int d = tid; d < kp.D; d += kFitThreads)
-            inl[d] = 0;
-        __syncthreads();
-        for (int j = tid; j < n; j += kFitThreads)
-            if (LD_IN(pid[j], kp.D, CK_FIT_ROW))
-                inl[pid[j]] = member[j];
         int flags = 0;
         if (fl & 1)
             flags |= LD_F_CAP_Y;
@@ -482,12 +518,17 @@ __device__ __forceinline__ void fit_body(const KParams &kp, const Work &w, const
             for (int i = 0; i < 3; ++i)
                 beta[i] = coef_s[i];
             // v_top: first row of the bottom run of rows with f(v) > 0 and f'(v) > 0
+            double fv[kPer], dfv[kPer];
             int worst = -1;
-            for (int v = tid; v < H; v += kFitThreads) {
+#pragma unroll
+            for (int i = 0; i < kPer; ++i) {
+                const int v = tid + i * kFitThreads;
+                if (v >= H)
+                    break;
                 const double tau = __dmul_rn((double)(v - centre), sc64);
-                const double fv = poly_f64<3>(beta, tau);
-                const double dfv = __dmul_rn(__dadd_rn(beta[1], __dmul_rn(__dmul_rn(2.0, beta[2]), tau)), sc64);
-                if (!(fv > 0.0 && dfv > 0.0))
+                fv[i] = poly_f64<3>(beta, tau);
+                dfv[i] = __dmul_rn(__dadd_rn(beta[1], __dmul_rn(__dmul_rn(2.0, beta[2]), tau)), sc64);
+                if (!(fv[i] > 0.0 && dfv[i] > 0.0))
                     worst = max(worst, v);
             }
             worst = __reduce_max_sync(0xffffffffu, worst);
@@ -502,14 +543,15 @@ __device__ __forceinline__ void fit_body(const KParams &kp, const Work &w, const
             }
             __syncthreads();
             vtop = sh[3];
-            for (int v = tid; v < H; v += kFitThreads) {
+#pragma unroll
+            for (int i = 0; i < kPer; ++i) {
+                const int v = tid + i * kFitThreads;
+                if (v >= H)
+                    break;
                 float F = 0.0f, Vy = 0.0f;
                 if (v >= vtop) {
-                    const double tau = __dmul_rn((double)(v - centre), sc64);
-                    const double fv = poly_f64<3>(beta, tau);
-                    const double dfv = __dmul_rn(__dadd_rn(beta[1], __dmul_rn(__dmul_rn(2.0, beta[2]), tau)), sc64);
-                    F = __double2float_rn(fv);
-                    Vy = __double2float_rn(__dsub_rn((double)v, __ddiv_rn(fv, dfv)));
+                    F = __double2float_rn(fv[i]);
+                    Vy = __double2float_rn(__dsub_rn((double)v, __ddiv_rn(fv[i], dfv[i])));
                 }
                 rows[v] = F;
                 rows[H + v] = Vy;
@@ -535,13 +577,6 @@ __device__ __forceinline__ void fit_body(const KParams &kp, const Work &w, const
                 fs.gamma[i] = 0.0;
         }
     } else {
-        uint8_t *inl = w.inl_x + (size_t)f * H;
-        for (int v = tid; v < H; v += kFitThreads)
-            inl[v] = 0;
-        __syncthreads();
-        for (int j = tid; j < n; j += kFitThreads)
-            if (LD_IN(pid[j], H, CK_FIT_ROW))
-                inl[pid[j]] = member[j];
         int flags = fs0.flags;
         if (fl & 1)
             flags |= LD_F_CAP_X;
@@ -577,20 +612,19 @@ __global__ void __launch_bounds__(kFitThreads) k_fit_fd(const FrameDesc *__restr
 }
 
 template <int M>
-size_t fit_smem(int P)
+size_t fit_smem(int P, int H)
 {
     size_t s = 0;
     auto add = [&](size_t bytes) { s = ((s + 15) & ~(size_t)15) + bytes; };
+    add(4 * (size_t)P);
+    add(8 * (size_t)P);
     add(2 * (size_t)P);
-    add(2 * (size_t)P);
-    add(2 * (size_t)P);
-    add((size_t)P);
-    add(2 * (size_t)P);
-    add(4 * (size_t)((P + 31) / 32 + 2));
+    add(4 * ((LD_MAX_H + kFitThreads - 1) / kFitThreads) * kNW);
     add(4 * kMaxHyps);
-    add(4 * kMaxHyps);
+    add(4 * (size_t)H);
     add(4 * kMaxHyps * 2 * M);
-    add(16 * kNW * (3 * M - 1));
+    add(16 * (3 * M - 1));
+    add(8 * kNW * (3 * M + 2));
     add(4 * kNW);
     return s + 16;
 }
@@ -611,25 +645,25 @@ cudaError_t setup_ransac(int smem_optin)
 
 cudaError_t launch_fit_y(const KParams &kp, const Work &w, cudaStream_t s)
 {
-    k_fit<3><<<kp.n_frames, kFitThreads, fit_smem<3>(w.pmax), s>>>(kp, w);
+    k_fit<3><<<kp.n_frames, kFitThreads, fit_smem<3>(w.pmax, kp.H), s>>>(kp, w);
     return cudaGetLastError();
 }
 
 cudaError_t launch_fit_y_fd(const KParams &kmax, const FrameDesc *fd, int n, cudaStream_t s)
 {
-    k_fit_fd<3><<<n, kFitThreads, fit_smem<3>(kmax.pmax_hint), s>>>(fd);
+    k_fit_fd<3><<<n, kFitThreads, fit_smem<3>(kmax.pmax_hint, kmax.H), s>>>(fd);
     return cudaGetLastError();
 }
 
 cudaError_t launch_fit_x_fd(const KParams &kmax, const FrameDesc *fd, int n, cudaStream_t s)
 {
-    k_fit_fd<5><<<n, kFitThreads, fit_smem<5>(kmax.pmax_hint), s>>>(fd);
+    k_fit_fd<5><<<n, kFitThreads, fit_smem<5>(kmax.pmax_hint, kmax.H), s>>>(fd);
     return cudaGetLastError();
 }
 
 cudaError_t launch_fit_x(const KParams &kp, const Work &w, cudaStream_t s)
 {
-    k_fit<5><<<kp.n_frames, kFitThreads, fit_smem<5>(w.pmax), s>>>(kp, w);
+    k_fit<5><<<kp.n_frames, kFitThreads, fit_smem<5>(w.pmax, kp.H), s>>>(kp, w);
     return cudaGetLastError();
 }
 
