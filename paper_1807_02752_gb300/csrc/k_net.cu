@@ -329,8 +329,20 @@ __global__ void __launch_bounds__(kConvThreads) k_conv_tc(const ConvIO io, int *
                     atomicExch(err, 1);
             }
             phase[pb] ^= 1u;
+        }
+        // the next tile's halo goes into the buffer the previous tile's MMAs have finished with, before that
+        // tile's epilogue, so that the copies run under it
+        const int done = prev;
+        prev = cur;
+        if (cur < total) {
+            cur = next_tile(cur + gridDim.x);
+            if (cur < total && ok)
+                load_halo(cur, halo[b ^ 1]);
+        }
+        if (done < total) {
+            const int pb = b ^ 1;
             asm volatile("tcgen05.fence::after_thread_sync;");
-            const int f = prev / per_frame, rem = prev % per_frame;
+            const int f = done / per_frame, rem = done % per_frame;
             const int y = (rem / io.tiles_c) * kTcRows + warp * 4 + (lane >> 3), x = (rem % io.tiles_c) * kTcCols + (lane & 7);
             uint32_t r[COUT];
             if (ok)
@@ -378,13 +390,6 @@ __global__ void __launch_bounds__(kConvThreads) k_conv_tc(const ConvIO io, int *
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;");
-        }
-        // the next tile's halo goes into the buffer the previous tile's MMAs have finished with
-        prev = cur;
-        if (cur < total) {
-            cur = next_tile(cur + gridDim.x);
-            if (cur < total && ok)
-                load_halo(cur, halo[b ^ 1]);
         }
         ++it;
     }
@@ -711,6 +716,18 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_net_fused(const FusedIO io
 
 // ---------------------------------------------------------------------------------------------------
 // weight gradients: dW[co][tap][ci] = sum_cells dS[co] A[cell + (tap)][ci]; column 9 CIN holds the bias
+//
+// Per tile of 8 x 16 cells the halo of A and the tile of dS sit in shared memory as the maps have them, a
+// cell's channels together, and both MMA operands come out of them with ldmatrix.trans: K is the cells, so
+// the transposing load of 8 cells x 8 channels is the fragment, for A at the tap's offset in the halo.
+// Cell strides of 2 C + 16 bytes keep the eight 16-byte rows of a matrix on different banks.  The 9 CIN / 16
+// groups of 16 columns are spread over the four warps (5 5 4 4 with the bias column on the last one's side,
+// or 3 2 2 2); the next tile arrives by cp.async into the other buffer while this one is multiplied.
+// kWgradCtasPerSm CTAs of 49 KB share an SM.
+// Bound by the tensor pipe's rate for warp-level MMAs (74 of them per 16 cells with 32 x 32 channels; the
+// maps would take 35 us at the copy bandwidth).  64 frames of 1242 x 375: 120 / 75 / 80 us for 32x32, 32->16
+// and 16->32 channels, and 28 us for the first layer; with B gathered element by element and the dS tile
+// transposed by its writers, one buffer, these took 260 / 214 / 176 / 72 us.
 // ---------------------------------------------------------------------------------------------------
 struct WgradIO {
     const __nv_bfloat16 *dS;     // [n][mh][mw][COUT]
@@ -722,112 +739,127 @@ struct WgradIO {
 template <int CIN, int COUT>
 struct WgradShape {
     static constexpr int NCOL = 9 * CIN + 1;
-    static constexpr int NTT = (NCOL + 7) / 8;          // n8 tiles
-    static constexpr int NPW = (NTT + 3) / 4;           // per warp
+    static constexpr int NG = 9 * CIN / 16;             // groups of 16 columns (two n8 tiles)
+    static constexpr int GPW = (NG + 3) / 4;            // per warp, at most
     static constexpr int MT = COUT / 16;
-    static constexpr int CINP = CIN == 1 ? 2 : CIN + 8; // halo cell stride (elements)
-    static constexpr int PXP = kTileR * kTileC + 8;     // dS^T row stride (elements)
-    static constexpr size_t bytes = sizeof(__nv_bfloat16) * (size_t)(kHaloR * kHaloC * CINP + COUT * PXP);
+    static constexpr int AS = CIN * 2 + 16;             // cell strides (bytes)
+    static constexpr int DS = COUT * 2 + 16;
+    static constexpr int abytes = kHaloR * kHaloC * AS, dbytes = kTileR * kTileC * DS;
+    static constexpr size_t bytes = 2 * (size_t)(abytes + dbytes);
+    static_assert(abytes % 16 == 0 && dbytes % 16 == 0, "16-byte aligned buffers");
 };
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool in)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
+}
+
+__device__ __forceinline__ void ldsm4_t(uint32_t (&r)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+
+// the dS cells of one tile into shared memory, zero outside the map
+template <int COUT>
+__device__ __forceinline__ void wgrad_load_ds(const WgradIO &io, int f, int y0, int x0, uint32_t dst)
+{
+    for (int i = threadIdx.x; i < kTileR * kTileC * (COUT / 8); i += kConvThreads) {
+        const int cell = i / (COUT / 8), ch = i % (COUT / 8);
+        const int yy = y0 + cell / kTileC, xx = x0 + cell % kTileC;
+        const bool in = yy < io.mh && xx < io.mw;
+        const size_t c = ((size_t)f * io.mh + (in ? yy : 0)) * io.mw + (in ? xx : 0);
+        cp_async16(dst + cell * (COUT * 2 + 16) + ch * 16, io.dS + c * COUT + ch * 8, in);
+    }
+}
+
+// A fragments (dS^T) of tile row r: matrices (cells 0-7 | 8-15) x (channels 0-7 | 8-15) per 16 channels
+template <int MT, int DS>
+__device__ __forceinline__ void wgrad_frag_a(uint32_t (&af)[MT][4], uint32_t sd, int r, int lane)
+{
+    const int cell = r * kTileC + ((lane >> 4) << 3) + (lane & 7);
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt)
+        ldsm4_t(af[mt], sd + cell * DS + mt * 32 + ((lane >> 3) & 1) * 16);
+}
 
 template <int CIN, int COUT>
 __global__ void __launch_bounds__(kConvThreads) k_wgrad(const WgradIO io)
 {
     using S = WgradShape<CIN, COUT>;
-    extern __shared__ __align__(16) __nv_bfloat16 gsm[];
-    __nv_bfloat16 *sA = gsm;                                   // [10 x 18][CINP]
-    __nv_bfloat16 *sD = gsm + kHaloR * kHaloC * S::CINP;        // [COUT][PXP]: dS transposed
-    const uint16_t *sA16 = reinterpret_cast<const uint16_t *>(sA);
+    extern __shared__ __align__(16) unsigned char gsm[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
     const int mh = io.mh, mw = io.mw;
     const int per_frame = io.tiles_r * io.tiles_c;
     const int total = io.n * per_frame;
-    // this lane's B column in each of the warp's n-tiles: (tap, ci), the bias column, or nothing
-    int coff[S::NPW];    // element offset of (dy, dx, ci) in the halo tile, -1 = zero column, -2 = ones
+    const uint32_t base = (uint32_t)__cvta_generic_to_shared(gsm);
+    // this warp's groups: the first NG % 4 warps have one more
+    constexpr int kLess = S::NG / 4, kMore = S::NG % 4;
+    const int g0 = warp * kLess + (warp < kMore ? warp : kMore), ng = kLess + (warp < kMore ? 1 : 0);
+    const bool has_bias = warp == 3;
+    const uint32_t ones = g == 0 ? 0x3f803f80u : 0u;   // the bias tile's only column
+    // lane's row of the B matrices: n-tile (lane >> 4), cells (lane >> 3 & 1) * 8 + (lane & 7)
+    uint32_t boff[S::GPW];
 #pragma unroll
-    for (int j = 0; j < S::NPW; ++j) {
-        const int col = (warp * S::NPW + j) * 8 + g;
-        if (col < 9 * CIN) {
-            const int tap = col / CIN, ci = col % CIN;
-            coff[j] = ((tap / 3) * kHaloC + tap % 3) * S::CINP + ci;
-        } else {
-            coff[j] = col == 9 * CIN ? -2 : -1;
-        }
+    for (int j = 0; j < S::GPW; ++j) {
+        const int col = (g0 + (j < ng ? j : 0)) * 16, tap = col / CIN, ci = col % CIN;
+        boff[j] = ((tap / 3) * kHaloC + tap % 3 + ((lane >> 3) & 1) * 8 + (lane & 7)) * S::AS + ci * 2 + (lane >> 4) * 16;
     }
-    float acc[S::MT][S::NPW][4];
+    float acc[S::MT][2 * S::GPW][4], accb[S::MT][4];
 #pragma unroll
-    for (int mt = 0; mt < S::MT; ++mt)
+    for (int mt = 0; mt < S::MT; ++mt) {
 #pragma unroll
-        for (int j = 0; j < S::NPW; ++j)
+        for (int q = 0; q < 4; ++q)
+            accb[mt][q] = 0.0f;
+#pragma unroll
+        for (int j = 0; j < 2 * S::GPW; ++j)
 #pragma unroll
             for (int q = 0; q < 4; ++q)
                 acc[mt][j][q] = 0.0f;
-    const uint16_t one = 0x3f80;   // bf16 1.0
-    for (int tile = blockIdx.x; tile < total; tile += gridDim.x) {
+    }
+    auto load_tile = [&](int tile, int buf) {
         const int f = tile / per_frame, rem = tile % per_frame;
         const int y0 = (rem / io.tiles_c) * kTileR, x0 = (rem % io.tiles_c) * kTileC;
-        __syncthreads();
-        if constexpr (CIN == 1) {
-            for (int i = tid; i < kHaloR * kHaloC; i += kConvThreads) {
-                const int yy = y0 - 1 + i / kHaloC, xx = x0 - 1 + i % kHaloC;
-                __nv_bfloat16 v = __float2bfloat16_rn(0.0f);
-                if (yy >= 0 && yy < mh && xx >= 0 && xx < mw)
-                    v = io.A[((size_t)f * mh + yy) * mw + xx];
-                sA[i * S::CINP] = v;
-            }
-        } else {
-            for (int i = tid; i < kHaloR * kHaloC * (CIN / 8); i += kConvThreads) {
-                const int cell = i / (CIN / 8), ch = i % (CIN / 8);
-                const int yy = y0 - 1 + cell / kHaloC, xx = x0 - 1 + cell % kHaloC;
-                uint4 v = make_uint4(0, 0, 0, 0);
-                if (yy >= 0 && yy < mh && xx >= 0 && xx < mw)
-                    v = __ldg(reinterpret_cast<const uint4 *>(io.A + (((size_t)f * mh + yy) * mw + xx) * CIN) + ch);
-                *reinterpret_cast<uint4 *>(sA + cell * S::CINP + ch * 8) = v;
-            }
+        const uint32_t sa = base + buf * (S::abytes + S::dbytes);
+        for (int i = tid; i < kHaloR * kHaloC * (CIN / 8); i += kConvThreads) {
+            const int cell = i / (CIN / 8), ch = i % (CIN / 8);
+            const int yy = y0 - 1 + cell / kHaloC, xx = x0 - 1 + cell % kHaloC;
+            const bool in = yy >= 0 && yy < mh && xx >= 0 && xx < mw;
+            const size_t c = ((size_t)f * mh + (in ? yy : 0)) * mw + (in ? xx : 0);
+            cp_async16(sa + cell * S::AS + ch * 16, io.A + c * CIN + ch * 8, in);
         }
-        // dS of the tile's 128 cells, transposed to [co][cell]; cells outside the map are 0
-        for (int i = tid; i < kTileR * kTileC * (COUT / 8); i += kConvThreads) {
-            const int cell = i / (COUT / 8), ch = i % (COUT / 8);
-            const int yy = y0 + cell / kTileC, xx = x0 + cell % kTileC;
-            uint4 v = make_uint4(0, 0, 0, 0);
-            if (yy < mh && xx < mw)
-                v = __ldg(reinterpret_cast<const uint4 *>(io.dS + (((size_t)f * mh + yy) * mw + xx) * COUT) + ch);
-            const uint16_t *e = reinterpret_cast<const uint16_t *>(&v);
-            uint16_t *col = reinterpret_cast<uint16_t *>(sD) + (ch * 8) * S::PXP + cell;
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-                col[k * S::PXP] = e[k];
-        }
-        __syncthreads();
-#pragma unroll 1
+        wgrad_load_ds<COUT>(io, f, y0, x0, sa + S::abytes);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    if ((int)blockIdx.x < total)
+        load_tile(blockIdx.x, 0);
+    int buf = 0;
+    for (int tile = blockIdx.x; tile < total; tile += gridDim.x, buf ^= 1) {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();   // this tile has landed for every thread, and the other buffer is read no more
+        if (tile + (int)gridDim.x < total)
+            load_tile(tile + gridDim.x, buf ^ 1);
+        const uint32_t sa = base + buf * (S::abytes + S::dbytes), sd = sa + S::abytes;
+#pragma unroll 2
         for (int r = 0; r < kTileR; ++r) {           // one k16 step per tile row (16 cells)
             uint32_t af[S::MT][4];
+            wgrad_frag_a<S::MT, S::DS>(af, sd, r, lane);
 #pragma unroll
-            for (int mt = 0; mt < S::MT; ++mt) {
-                const __nv_bfloat16 *r0 = sD + (mt * 16 + g) * S::PXP + r * kTileC + 2 * t;
-                const __nv_bfloat16 *r1 = r0 + 8 * S::PXP;
-                af[mt][0] = *reinterpret_cast<const uint32_t *>(r0);
-                af[mt][1] = *reinterpret_cast<const uint32_t *>(r1);
-                af[mt][2] = *reinterpret_cast<const uint32_t *>(r0 + 8);
-                af[mt][3] = *reinterpret_cast<const uint32_t *>(r1 + 8);
-            }
-            const int rowoff = r * kHaloC * S::CINP;
-#pragma unroll
-            for (int j = 0; j < S::NPW; ++j) {
-                if ((warp * S::NPW + j) * 8 >= S::NCOL)
+            for (int j = 0; j < S::GPW; ++j) {
+                if (j >= kLess && j >= ng)
                     break;
-                uint32_t b0, b1;
-                if (coff[j] >= 0) {
-                    const uint16_t *p = sA16 + rowoff + coff[j] + (2 * t) * S::CINP;
-                    b0 = pack_raw(p[0], p[S::CINP]);
-                    b1 = pack_raw(p[8 * S::CINP], p[9 * S::CINP]);
-                } else {
-                    b0 = coff[j] == -2 ? pack_raw(one, one) : 0u;
-                    b1 = b0;
+                uint32_t b[4];
+                ldsm4_t(b, sa + r * kHaloC * S::AS + boff[j]);
+#pragma unroll
+                for (int mt = 0; mt < S::MT; ++mt) {
+                    mma16816(acc[mt][2 * j], af[mt][0], af[mt][1], af[mt][2], af[mt][3], b[0], b[1]);
+                    mma16816(acc[mt][2 * j + 1], af[mt][0], af[mt][1], af[mt][2], af[mt][3], b[2], b[3]);
                 }
+            }
+            if (has_bias) {
 #pragma unroll
                 for (int mt = 0; mt < S::MT; ++mt)
-                    mma16816(acc[mt][j], af[mt][0], af[mt][1], af[mt][2], af[mt][3], b0, b1);
+                    mma16816(accb[mt], af[mt][0], af[mt][1], af[mt][2], af[mt][3], ones, ones);
             }
         }
     }
@@ -835,27 +867,122 @@ __global__ void __launch_bounds__(kConvThreads) k_wgrad(const WgradIO io)
 #pragma unroll
     for (int mt = 0; mt < S::MT; ++mt)
 #pragma unroll
-        for (int j = 0; j < S::NPW; ++j) {
-            const int c0 = (warp * S::NPW + j) * 8 + 2 * t;
+        for (int q = 0; q < 4; ++q) {
+            float *row = part + (mt * 16 + g + (q >> 1) * 8) * S::NCOL;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int co = mt * 16 + g + (q >> 1) * 8, col = c0 + (q & 1);
-                if (col < S::NCOL)
-                    part[co * S::NCOL + col] = acc[mt][j][q];
-            }
+            for (int j = 0; j < 2 * S::GPW; ++j)
+                if ((j >> 1) < ng)
+                    row[g0 * 16 + j * 8 + 2 * t + (q & 1)] = acc[mt][j][q];
+            if (has_bias && t == 0 && (q & 1) == 0)
+                row[9 * CIN] = accb[mt][q];
         }
 }
 
-// Sum the per-CTA partials in CTA order and scatter into the flat gradient (layout [co][ci][3][3], b[co]).
-__global__ void k_wreduce(const float *part, int nparts, int cin, int cout, float *grad_w, float *grad_b)
+// The first layer (one input channel): ten columns (nine taps and the bias) in two n-tiles, so the warps
+// split the cells instead, two tile rows each, and their sums are added in warp order at the end.
+__global__ void __launch_bounds__(kConvThreads) k_wgrad1(const WgradIO io)
+{
+    constexpr int COUT = 16, DS = COUT * 2 + 16, kHalo = kHaloR * kHaloC, kPer = (kHalo + kConvThreads - 1) / kConvThreads;
+    __shared__ __align__(16) unsigned char sd_raw[2][kTileR * kTileC * DS];
+    __shared__ uint16_t sa[2][kHalo];
+    __shared__ float red[4][COUT][10];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+    const int mh = io.mh, mw = io.mw, per_frame = io.tiles_r * io.tiles_c, total = io.n * per_frame;
+    const uint32_t dbase = (uint32_t)__cvta_generic_to_shared(&sd_raw[0][0]);
+    const uint16_t *A = reinterpret_cast<const uint16_t *>(io.A);
+    uint16_t next[kPer];
+    auto load_tile = [&](int tile, int buf) {
+        const int f = tile / per_frame, rem = tile % per_frame;
+        const int y0 = (rem / io.tiles_c) * kTileR, x0 = (rem % io.tiles_c) * kTileC;
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+            const int i = tid + k * kConvThreads, yy = y0 - 1 + i / kHaloC, xx = x0 - 1 + i % kHaloC;
+            next[k] = 0;
+            if (i < kHalo && yy >= 0 && yy < mh && xx >= 0 && xx < mw)
+                next[k] = __ldg(A + ((size_t)f * mh + yy) * mw + xx);
+        }
+        wgrad_load_ds<COUT>(io, f, y0, x0, dbase + buf * (kTileR * kTileC * DS));
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float acc[1][2][4] = {};
+    const int tapoff = (g / 3) * kHaloC + g % 3;   // tap g, columns 0-7 of the first n-tile
+    const uint32_t ones = g == 1 ? 0x3f803f80u : 0u;
+    if ((int)blockIdx.x < total)
+        load_tile(blockIdx.x, 0);
+    int buf = 0;
+    for (int tile = blockIdx.x; tile < total; tile += gridDim.x, buf ^= 1) {
+#pragma unroll
+        for (int k = 0; k < kPer; ++k)
+            if (tid + k * kConvThreads < kHalo)
+                sa[buf][tid + k * kConvThreads] = next[k];
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        if (tile + (int)gridDim.x < total)
+            load_tile(tile + gridDim.x, buf ^ 1);
+#pragma unroll
+        for (int rr = 0; rr < 2; ++rr) {
+            const int r = warp * 2 + rr;
+            uint32_t af[1][4];
+            wgrad_frag_a<1, DS>(af, dbase + buf * (kTileR * kTileC * DS), r, lane);
+            const uint16_t *p = &sa[buf][r * kHaloC + tapoff + 2 * t];
+            mma16816(acc[0][0], af[0][0], af[0][1], af[0][2], af[0][3], pack_raw(p[0], p[1]), pack_raw(p[8], p[9]));
+            // second n-tile: tap 8 (halo offset 2 rows, 2 columns) in column 0, ones in column 1
+            const uint16_t *p8 = &sa[buf][(r + 2) * kHaloC + 2 + 2 * t];
+            const uint32_t b0 = g == 0 ? pack_raw(p8[0], p8[1]) : ones, b1 = g == 0 ? pack_raw(p8[8], p8[9]) : ones;
+            mma16816(acc[0][1], af[0][0], af[0][1], af[0][2], af[0][3], b0, b1);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int co = g + (q >> 1) * 8, c = 2 * t + (q & 1);
+        red[warp][co][c] = acc[0][0][q];
+        if (c < 2)
+            red[warp][co][8 + c] = acc[0][1][q];
+    }
+    __syncthreads();
+    for (int i = tid; i < COUT * 10; i += kConvThreads) {
+        const float *r0 = &red[0][0][0] + i;
+        io.part[(size_t)blockIdx.x * COUT * 10 + i] =
+            __fadd_rn(__fadd_rn(r0[0], r0[COUT * 10]), __fadd_rn(r0[2 * COUT * 10], r0[3 * COUT * 10]));
+    }
+}
+
+// Sum of nparts partials [nparts][stride] per output, in a fixed order: slice s of a block adds partials
+// s, s + slices, ..., then the slices are added by halves.  32 outputs (a 128-byte line of a partial) x 32
+// slices per block; the sum is on slice 0's threads.  608 partials: 7-8 us a layer (22 MB for the widest, from
+// L2) against 51-56 us with one thread adding all partials of an output one after another; the loss 6 us
+// against 22.
+constexpr int kRedSlices = 32;
+
+__device__ __forceinline__ float sum_partials(const float *part, int nparts, int stride, int i, bool in)
+{
+    __shared__ float red[kRedSlices][33];
+    const int o = threadIdx.x & 31, sl = threadIdx.x >> 5;
+    float s = 0.0f;
+    if (in) {
+#pragma unroll 4
+        for (int k = sl; k < nparts; k += kRedSlices)
+            s = __fadd_rn(s, part[(size_t)k * stride + i]);
+    }
+    red[sl][o] = s;
+    for (int h = kRedSlices / 2; h > 0; h >>= 1) {
+        __syncthreads();
+        if (sl < h)
+            red[sl][o] = s = __fadd_rn(s, red[sl + h][o]);
+    }
+    return s;
+}
+
+// The per-CTA partials of a layer, summed and scattered into the flat gradient (layout [co][ci][3][3], b[co]).
+__global__ void __launch_bounds__(32 * kRedSlices) k_wreduce(const float *part, int nparts, int cin, int cout,
+                                                             float *grad_w, float *grad_b)
 {
     const int ncol = 9 * cin + 1;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= cout * ncol)
+    const int i = blockIdx.x * 32 + (threadIdx.x & 31);
+    const bool in = i < cout * ncol;
+    const float s = sum_partials(part, nparts, cout * ncol, i, in);
+    if (!in || threadIdx.x >= 32)
         return;
-    float s = 0.0f;
-    for (int k = 0; k < nparts; ++k)
-        s = __fadd_rn(s, part[(size_t)k * cout * ncol + i]);
     const int co = i / ncol, col = i % ncol;
     if (col == 9 * cin)
         grad_b[co] = s;
@@ -937,14 +1064,13 @@ __global__ void __launch_bounds__(kCellThreads) k_loss(const NetArgs a, const ui
 }
 
 // loss and the head's gradient from the k_loss partials (fixed order)
-__global__ void k_loss_reduce(const float *part, int nparts, float inv_n, float *grad_head, float *loss_out)
+__global__ void __launch_bounds__(32 * kRedSlices) k_loss_reduce(const float *part, int nparts, float inv_n,
+                                                                 float *grad_head, float *loss_out)
 {
-    const int k = threadIdx.x;
-    if (k >= 18)
+    const int k = threadIdx.x & 31;
+    const float s = sum_partials(part, nparts, 18, k, k < 18);
+    if (k >= 18 || threadIdx.x >= 32)
         return;
-    float s = 0.0f;
-    for (int i = 0; i < nparts; ++i)
-        s = __fadd_rn(s, part[(size_t)i * 18 + k]);
     if (k == 0) {
         if (loss_out)
             *loss_out = s * inv_n;
@@ -1328,12 +1454,25 @@ static cudaError_t wgrad(const NetArgs &a, const __nv_bfloat16 *dS, const __nv_b
     io.tiles_r = (a.mh + kTileR - 1) / kTileR;
     io.tiles_c = (a.mw + kTileC - 1) / kTileC;
     const int G = grid_for(n * io.tiles_r * io.tiles_c, kWgradCtasPerSm);
-    k_wgrad<CIN, COUT><<<G, kConvThreads, WgradShape<CIN, COUT>::bytes, s>>>(io);
+    if constexpr (CIN == 1) {
+        static_assert(COUT == 16, "k_wgrad1 is the first layer's");
+        k_wgrad1<<<G, kConvThreads, 0, s>>>(io);
+    } else {
+        static bool attr = false;
+        if (!attr) {
+            cudaError_t e = cudaFuncSetAttribute(k_wgrad<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)WgradShape<CIN, COUT>::bytes);
+            if (e != cudaSuccess)
+                return e;
+            attr = true;
+        }
+        k_wgrad<CIN, COUT><<<G, kConvThreads, WgradShape<CIN, COUT>::bytes, s>>>(io);
+    }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
         return e;
     const int outs = COUT * (9 * CIN + 1);
-    k_wreduce<<<(outs + 255) / 256, 256, 0, s>>>(a.part, G, CIN, COUT, gw, gb);
+    k_wreduce<<<(outs + 31) / 32, 32 * kRedSlices, 0, s>>>(a.part, G, CIN, COUT, gw, gb);
     return cudaGetLastError();
 }
 
@@ -1348,7 +1487,7 @@ cudaError_t net_backward(const NetArgs &a, const uint8_t *labels, int n, float p
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
         return e;
-    k_loss_reduce<<<1, 32, 0, s>>>(a.part_head, GL, inv_n, grad + kNetParams - 17, loss);
+    k_loss_reduce<<<1, 32 * kRedSlices, 0, s>>>(a.part_head, GL, inv_n, grad + kNetParams - 17, loss);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return e;
     // parameter offsets
