@@ -57,6 +57,25 @@ __device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool in)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
+}
+
+// 32 bytes of a cell at once (a whole sector; the maps' cells are 32 or 64 bytes from a 256-byte aligned base)
+__device__ __forceinline__ void ld_cell32(uint32_t (&r)[8], const void *p)
+{
+    asm volatile("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "l"(p));
+}
+
+__device__ __forceinline__ void st_cell32(void *p, const uint32_t (&r)[8])
+{
+    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                 ::"l"(p), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
+}
+
 // first cell row a layer must produce for frame f, or INT_MAX when the frame needs nothing
 __device__ __forceinline__ int first_needed_row(const FrameState *fs, int f, int depth)
 {
@@ -76,47 +95,56 @@ __device__ __forceinline__ float cell_input(int32_t s)
 
 // ---------------------------------------------------------------------------------------------------
 // layer 1: one input channel, K = 9, direct FMA per cell
+//
+// Bound by the cells' instructions (the maps take 10 us): the weights are read four channels at a time and
+// multiplied in channel pairs, which halves both.  64 frames of 1242 x 375: 26 us (one weight per load, one
+// channel per FMA and 64-bit cell arithmetic: 41 us).
 // ---------------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kCellThreads) k_conv1(const NetArgs a, const int32_t *xsum, int n,
                                                         const FrameState *fs)
 {
-    __shared__ float wsm[16 * 9 + 16];
+    __shared__ __align__(16) float wsm[9 * 16 + 16];   // [tap][co], then the bias
     for (int i = threadIdx.x; i < 16 * 9; i += kCellThreads)
-        wsm[i] = __bfloat162float(a.wf[0][i]);   // [co][tap]
+        wsm[(i % 9) * 16 + i / 9] = __bfloat162float(a.wf[0][i]);   // [co][tap]
     for (int i = threadIdx.x; i < 16; i += kCellThreads)
         wsm[144 + i] = a.bias[0][i];
     __syncthreads();
-    const int mh = a.mh, mw = a.mw;
-    const long long cells = (long long)n * mh * mw;
-    for (long long p = blockIdx.x * (long long)kCellThreads + threadIdx.x; p < cells;
-         p += (long long)gridDim.x * kCellThreads) {
-        const int x = (int)(p % mw);
-        const int y = (int)((p / mw) % mh);
-        const long long fb = p - (long long)y * mw - x;   // first cell of the frame
-        if (y < first_needed_row(fs, (int)(p / ((long long)mh * mw)), 3))
+    const uint32_t mh = a.mh, mw = a.mw, cells = n * mh * mw;   // fewer than 2^31: a cell holds over 160 bytes
+    for (uint32_t p = blockIdx.x * kCellThreads + threadIdx.x; p < cells; p += gridDim.x * kCellThreads) {
+        const uint32_t row = p / mw, f = row / mh;
+        const int x = (int)(p - row * mw), y = (int)(row - f * mh);
+        if (y < first_needed_row(fs, (int)f, 3))
             continue;
+        const int32_t *src = xsum + p;
         float in[9];
 #pragma unroll
         for (int t = 0; t < 9; ++t) {
-            const int yy = y + t / 3 - 1, xx = x + t % 3 - 1;
-            in[t] = (yy >= 0 && yy < mh && xx >= 0 && xx < mw) ? cell_input(__ldg(xsum + fb + (long long)yy * mw + xx)) : 0.0f;
+            const int dy = t / 3 - 1, dx = t % 3 - 1;
+            const bool ok = (unsigned)(y + dy) < mh && (unsigned)(x + dx) < mw;
+            in[t] = ok ? cell_input(__ldg(src + dy * (int)mw + dx)) : 0.0f;
         }
         if (a.X)
             a.X[p] = __float2bfloat16_rn(in[4]);
+        float2 acc[8];   // channel pairs: each half is one correctly rounded fused step, taps in order
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            acc[c] = reinterpret_cast<const float2 *>(wsm + 144)[c];
+#pragma unroll
+        for (int t = 0; t < 9; ++t) {
+            const float2 v = make_float2(in[t], in[t]);
+            const float4 *wt = reinterpret_cast<const float4 *>(wsm + t * 16);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float4 w4 = wt[c];
+                acc[2 * c] = __ffma2_rn(make_float2(w4.x, w4.y), v, acc[2 * c]);
+                acc[2 * c + 1] = __ffma2_rn(make_float2(w4.z, w4.w), v, acc[2 * c + 1]);
+            }
+        }
         uint32_t o[8];
 #pragma unroll
-        for (int c = 0; c < 16; c += 2) {
-            float s0 = wsm[144 + c], s1 = wsm[144 + c + 1];
-#pragma unroll
-            for (int t = 0; t < 9; ++t) {
-                s0 = __fmaf_rn(wsm[c * 9 + t], in[t], s0);
-                s1 = __fmaf_rn(wsm[(c + 1) * 9 + t], in[t], s1);
-            }
-            o[c >> 1] = pack2(fmaxf(s0, 0.0f), fmaxf(s1, 0.0f));
-        }
-        uint4 *dst = reinterpret_cast<uint4 *>(a.act[0] + p * 16);
-        dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
-        dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
+        for (int c = 0; c < 8; ++c)
+            o[c] = pack2(fmaxf(acc[c].x, 0.0f), fmaxf(acc[c].y, 0.0f));
+        st_cell32(a.act[0] + (size_t)p * 16, o);
     }
 }
 
@@ -156,20 +184,29 @@ struct ConvIO {
 // C_out x 16 B apart, groups of 8 output channels 128 B apart.  One thread issues the 9 C_in / 16 MMAs of a
 // tile (M 128, N C_out, K 16, bf16 -> f32) into one of two accumulators in tensor memory and commits them to
 // an mbarrier; meanwhile the CTA reads the other accumulator (tcgen05.ld, one tensor-memory lane quarter per
-// warp: a thread gets all C_out channels of one cell) for the previous tile's epilogue and copies the next
-// tile's halo in with cp.async (zero-filled outside the map).  Waits are bounded: on a timeout the kernel
-// records it in err and stops issuing work.
+// warp: a thread gets all C_out channels of one cell) for the previous tile's epilogue and copies the halo of
+// the tile after the next in with cp.async (zero-filled outside the map).  Waits are bounded: on a timeout the
+// kernel records it in err and stops issuing work.
+//
+// Bound by latency: a tile's halo, MMAs and epilogue depend on one another, so three halo buffers keep two
+// tiles' copies in flight, a warp of its own issues the MMAs (the issuing thread is held up while the queue is
+// full and would hold up its warp's epilogue), a warp copies and stores whole cells (32-byte sectors), and the
+// mask of the backward pass is fetched before the wait for the MMAs.  64 frames of 1242 x 375, 16->32 / 32->32
+// / 32->16 channels: forward 56 / 79 / 83 us, backward 80 / 98 / 75 us (us at the copy bandwidth: 27 / 35 / 27
+// and 35 / 53 / 44); with two buffers, no issuing warp and 16-byte pieces 70 / 104 / 98 and 100 / 134 / 115.
 // ---------------------------------------------------------------------------------------------------
 constexpr int kTcRows = 16, kTcCols = 8;                       // output tile (cells)
 constexpr int kTcHR = kTcRows + 2, kTcHC = kTcCols + 2;         // halo
 constexpr int kTcPlane = kTcHR * kTcHC * 16;                    // bytes of one 8-channel plane of the halo
+constexpr int kTcStages = 3;                                    // halo buffers: one multiplied, two on their way
+constexpr int kTcThreads = kConvThreads + 32;                   // copying and epilogue warps, and the issuing one
 constexpr unsigned kTcSpin = 1u << 26;                           // wait limit (iterations)
 
 template <int CIN, int COUT>
 struct TcSmem {
     static constexpr int halo = (CIN / 8) * kTcPlane;            // one halo buffer
     static constexpr int wts = 9 * CIN * COUT * 2;               // B operand, all taps
-    static constexpr size_t bytes = 2 * (size_t)halo + wts + 128;
+    static constexpr size_t bytes = kTcStages * (size_t)halo + wts;
 };
 
 __device__ __forceinline__ uint64_t tc_desc(uint32_t addr, uint32_t lbo, uint32_t sbo)
@@ -218,20 +255,20 @@ __device__ __forceinline__ void tc_load<32>(uint32_t taddr, uint32_t (&r)[32])
 }
 
 template <int CIN, int COUT, int EPI>
-__global__ void __launch_bounds__(kConvThreads) k_conv_tc(const ConvIO io, int *err)
+__global__ void __launch_bounds__(kTcThreads) k_conv_tc(const ConvIO io, int *err)
 {
     using S = TcSmem<CIN, COUT>;
     extern __shared__ __align__(1024) unsigned char tsm_raw[];
     __shared__ uint32_t taddr_s;
     __shared__ __align__(8) uint64_t mbar[2];
-    unsigned char *halo[2] = {tsm_raw, tsm_raw + S::halo};
-    unsigned char *wsm = tsm_raw + 2 * S::halo;
+    __shared__ int stop;                      // a wait ran out: no more MMAs are issued
+    unsigned char *wsm = tsm_raw + kTcStages * S::halo;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int mh = io.mh, mw = io.mw;
     const int per_frame = io.tiles_r * io.tiles_c, total = io.n * per_frame;
     // weights -> B layout: K step kk = tap (CIN/16) + c16, half h: 16-byte row n at
     // kk (COUT 32) + h (COUT 16) + (n / 8) 128 + (n % 8) 16; a row holds the 8 input channels c16 16 + 8 h ..
-    for (int i = tid; i < COUT * 9 * (CIN / 8); i += kConvThreads) {
+    for (int i = tid; i < COUT * 9 * (CIN / 8); i += kTcThreads) {
         const int n = i / (9 * CIN / 8), rem = i % (9 * CIN / 8), tap = rem / (CIN / 8), c8 = rem % (CIN / 8);
         const int kk = tap * (CIN / 16) + (c8 >> 1), h = c8 & 1;
         const uint4 v = __ldg(reinterpret_cast<const uint4 *>(io.wt + (size_t)n * 9 * CIN + tap * CIN + c8 * 8));
@@ -239,6 +276,7 @@ __global__ void __launch_bounds__(kConvThreads) k_conv_tc(const ConvIO io, int *
     }
     const uint32_t mb0 = (uint32_t)__cvta_generic_to_shared(&mbar[0]), mb1 = (uint32_t)__cvta_generic_to_shared(&mbar[1]);
     if (tid == 0) {
+        stop = 0;
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb0));
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb1));
         asm volatile("fence.mbarrier_init.release.cluster;");
@@ -265,14 +303,12 @@ __global__ void __launch_bounds__(kConvThreads) k_conv_tc(const ConvIO io, int *
         const int f = t / per_frame, rem = t % per_frame;
         const int y0 = (rem / io.tiles_c) * kTcRows - 1, x0 = (rem % io.tiles_c) * kTcCols - 1;
         for (int i = tid; i < kTcHR * kTcHC * (CIN / 8); i += kConvThreads) {
-            const int p = i / (kTcHR * kTcHC), cell = i % (kTcHR * kTcHC);
+            const int p = i % (CIN / 8), cell = i / (CIN / 8);   // a warp reads whole cells: full sectors
             const int yy = y0 + cell / kTcHC, xx = x0 + cell % kTcHC;
             const bool in = yy >= 0 && yy < mh && xx >= 0 && xx < mw;
             const __nv_bfloat16 *src = io.in + (((size_t)f * mh + (in ? yy : 0)) * mw + (in ? xx : 0)) * CIN + p * 8;
-            const uint32_t dst = (uint32_t)__cvta_generic_to_shared(buf + p * kTcPlane + cell * 16);
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
+            cp_async16((uint32_t)__cvta_generic_to_shared(buf + p * kTcPlane + cell * 16), src, in);
         }
-        asm volatile("cp.async.commit_group;" ::: "memory");
     };
     float hw[16], bias[COUT];
     if (EPI == kEpiHead) {
@@ -288,21 +324,30 @@ __global__ void __launch_bounds__(kConvThreads) k_conv_tc(const ConvIO io, int *
     constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(COUT >> 3) << 17) | ((128u >> 4) << 24);
     const uint32_t wbase = (uint32_t)__cvta_generic_to_shared(wsm);
     bool ok = true;
-    int cur = next_tile(blockIdx.x), prev = total, it = 0;
+    const bool issuer = warp == kConvThreads / 32;
+    int cur = next_tile(blockIdx.x), nxt = cur < total ? next_tile(cur + gridDim.x) : total, prev = total;
     uint32_t phase[2] = {0u, 0u};
-    if (cur < total)
-        load_halo(cur, halo[0]);
-    while (cur < total || prev < total) {
+    if (!issuer) {
+        if (cur < total)
+            load_halo(cur, tsm_raw);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        if (nxt < total)
+            load_halo(nxt, tsm_raw + S::halo);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    for (int it = 0, st = 0; cur < total || prev < total; ++it) {
         const int b = it & 1;
         if (cur < total) {
-            // the halo of `cur` has landed: make it visible to the tensor cores and issue its MMAs
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            // the halo of `cur` has landed (the next one may be on its way): make it visible to the tensor
+            // cores and issue its MMAs
+            if (!issuer)
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             asm volatile("tcgen05.fence::before_thread_sync;");
             __syncthreads();
             asm volatile("tcgen05.fence::after_thread_sync;");
-            if (tid == 0 && ok) {
-                const uint32_t hbase = (uint32_t)__cvta_generic_to_shared(halo[b]);
+            if (tid == kConvThreads && !*(volatile int *)&stop) {
+                const uint32_t hbase = (uint32_t)__cvta_generic_to_shared(tsm_raw + st * S::halo);
                 const uint32_t dacc = tbase + (uint32_t)(b * 32);
 #pragma unroll
                 for (int tap = 0; tap < 9; ++tap)
@@ -320,68 +365,73 @@ __global__ void __launch_bounds__(kConvThreads) k_conv_tc(const ConvIO io, int *
                              ::"r"(b ? mb1 : mb0) : "memory");
             }
         }
-        if (prev < total) {
-            // the previous tile: wait for its MMAs, then read its accumulator and store the cells
-            const int pb = b ^ 1;
+        const int nn = nxt < total ? next_tile(nxt + gridDim.x) : total;
+        const int pst = st == 0 ? kTcStages - 1 : st - 1;   // the previous tile's buffer
+        const int pb = b ^ 1;
+        size_t cell = 0;                      // this thread's cell of the previous tile
+        bool inside = false;
+        uint32_t mk[EPI == kEpiMask ? COUT / 16 : 1][8];
+        if (prev < total && !issuer) {
+            // the previous tile: its mask is fetched while its MMAs are waited for
+            const int f = prev / per_frame, rem = prev % per_frame;
+            const int y = (rem / io.tiles_c) * kTcRows + warp * 4 + (lane >> 3), x = (rem % io.tiles_c) * kTcCols + (lane & 7);
+            inside = y < mh && x < mw;
+            cell = ((size_t)f * mh + y) * mw + x;
+            if (EPI == kEpiMask && inside) {
+#pragma unroll
+                for (int q = 0; q < COUT / 16; ++q)
+                    ld_cell32(mk[q], io.mask + cell * COUT + q * 16);
+            }
             if (ok && !__all_sync(0xffffffffu, tc_wait(pb ? mb1 : mb0, phase[pb]))) {
                 ok = false;   // uniform over the warp (tcgen05.ld is a warp-wide instruction)
-                if (lane == 0)
+                if (lane == 0) {
+                    *(volatile int *)&stop = 1;
                     atomicExch(err, 1);
+                }
             }
             phase[pb] ^= 1u;
         }
-        // the next tile's halo goes into the buffer the previous tile's MMAs have finished with, before that
-        // tile's epilogue, so that the copies run under it
-        const int done = prev;
-        prev = cur;
-        if (cur < total) {
-            cur = next_tile(cur + gridDim.x);
-            if (cur < total && ok)
-                load_halo(cur, halo[b ^ 1]);
+        if (!issuer) {
+            // the tile after the next goes into the buffer the previous tile's MMAs have finished with
+            if (nn < total && ok)
+                load_halo(nn, tsm_raw + pst * S::halo);
+            asm volatile("cp.async.commit_group;" ::: "memory");
         }
-        if (done < total) {
-            const int pb = b ^ 1;
+        if (prev < total && !issuer) {
+            // read the previous tile's accumulator and store its cells
             asm volatile("tcgen05.fence::after_thread_sync;");
-            const int f = done / per_frame, rem = done % per_frame;
-            const int y = (rem / io.tiles_c) * kTcRows + warp * 4 + (lane >> 3), x = (rem % io.tiles_c) * kTcCols + (lane & 7);
             uint32_t r[COUT];
             if (ok)
                 tc_load<COUT>(tbase + (uint32_t)(pb * 32) + ((uint32_t)(warp * 32) << 16), r);
-            if (ok && y < mh && x < mw) {
-                const size_t cell = ((size_t)f * mh + y) * mw + x;
+            if (ok && inside) {
                 if (EPI == kEpiMask) {
-                    const uint4 *mk = reinterpret_cast<const uint4 *>(io.mask + cell * COUT);
-                    uint4 *dst = reinterpret_cast<uint4 *>(io.out + cell * COUT);
 #pragma unroll
-                    for (int q = 0; q < COUT / 8; ++q) {
-                        const uint4 m4 = __ldg(mk + q);
-                        const uint32_t mw4[4] = {m4.x, m4.y, m4.z, m4.w};
-                        uint32_t o[4];
+                    for (int q = 0; q < COUT / 16; ++q) {
+                        uint32_t o[8];
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const float v0 = bf_lo(mw4[k]) > 0.0f ? __uint_as_float(r[q * 8 + 2 * k]) : 0.0f;
-                            const float v1 = bf_hi(mw4[k]) > 0.0f ? __uint_as_float(r[q * 8 + 2 * k + 1]) : 0.0f;
+                        for (int k = 0; k < 8; ++k) {
+                            const float v0 = bf_lo(mk[q][k]) > 0.0f ? __uint_as_float(r[q * 16 + 2 * k]) : 0.0f;
+                            const float v1 = bf_hi(mk[q][k]) > 0.0f ? __uint_as_float(r[q * 16 + 2 * k + 1]) : 0.0f;
                             o[k] = pack2(v0, v1);
                         }
-                        dst[q] = make_uint4(o[0], o[1], o[2], o[3]);
+                        st_cell32(io.out + cell * COUT + q * 16, o);
                     }
                 } else {
                     float zc = 0.0f;
-                    uint4 *dst = io.out ? reinterpret_cast<uint4 *>(io.out + cell * COUT) : nullptr;
 #pragma unroll
-                    for (int q = 0; q < COUT / 8; ++q) {
-                        uint32_t o[4];
+                    for (int q = 0; q < COUT / 16; ++q) {
+                        uint32_t o[8];
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const int c = q * 8 + 2 * k;
+                        for (int k = 0; k < 8; ++k) {
+                            const int c = q * 16 + 2 * k;
                             const float v0 = fmaxf(__fadd_rn(__uint_as_float(r[c]), bias[c]), 0.0f);
                             const float v1 = fmaxf(__fadd_rn(__uint_as_float(r[c + 1]), bias[c + 1]), 0.0f);
                             o[k] = pack2(v0, v1);
                             if (EPI == kEpiHead)
                                 zc = __fmaf_rn(hw[c + 1], bf_hi(o[k]), __fmaf_rn(hw[c], bf_lo(o[k]), zc));
                         }
-                        if (dst)
-                            dst[q] = make_uint4(o[0], o[1], o[2], o[3]);
+                        if (io.out)
+                            st_cell32(io.out + cell * COUT + q * 16, o);
                     }
                     if (EPI == kEpiHead) {
                         zc = __fadd_rn(zc, io.bh[0]);
@@ -391,7 +441,10 @@ __global__ void __launch_bounds__(kConvThreads) k_conv_tc(const ConvIO io, int *
             }
             asm volatile("tcgen05.fence::before_thread_sync;");
         }
-        ++it;
+        prev = cur;
+        cur = nxt;
+        nxt = nn;
+        st = st == kTcStages - 1 ? 0 : st + 1;
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;");
@@ -749,11 +802,6 @@ struct WgradShape {
     static_assert(abytes % 16 == 0 && dbytes % 16 == 0, "16-byte aligned buffers");
 };
 
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool in)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
-}
-
 __device__ __forceinline__ void ldsm4_t(uint32_t (&r)[4], uint32_t addr)
 {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
@@ -1010,9 +1058,8 @@ __global__ void __launch_bounds__(kCellThreads) k_loss(const NetArgs a, const ui
         acc[k] = 0.0f;
     for (long long p = blockIdx.x * (long long)kCellThreads + threadIdx.x; p < cells;
          p += (long long)gridDim.x * kCellThreads) {
-        const uint4 *src = reinterpret_cast<const uint4 *>(a.act[3] + p * 16);
-        const uint4 q0 = src[0], q1 = src[1];
-        const uint32_t w32[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
+        uint32_t w32[8];
+        ld_cell32(w32, a.act[3] + p * 16);
         float av[16];
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
@@ -1041,9 +1088,7 @@ __global__ void __launch_bounds__(kCellThreads) k_loss(const NetArgs a, const ui
             acc[2 + c] = __fmaf_rn(dz, av[c + 1], acc[2 + c]);
         }
         acc[17] += dz;
-        uint4 *dst = reinterpret_cast<uint4 *>(a.dS[0] + p * 16);
-        dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
-        dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
+        st_cell32(a.dS[0] + p * 16, o);
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -1357,7 +1402,7 @@ static cudaError_t conv(ConvIO io, cudaStream_t s)
     if (e != cudaSuccess)
         return e;
     const int tiles = io.n * io.tiles_r * io.tiles_c;
-    k_conv_tc<CIN, COUT, EPI><<<grid_for(tiles, 4), kConvThreads, S::bytes, s>>>(io, err);
+    k_conv_tc<CIN, COUT, EPI><<<grid_for(tiles, 4), kTcThreads, S::bytes, s>>>(io, err);
     return cudaGetLastError();
 }
 
