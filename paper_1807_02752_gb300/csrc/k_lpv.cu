@@ -24,7 +24,7 @@ namespace {
 
 constexpr int kM1Threads = 512;
 constexpr int kEnThreads = 128;
-constexpr int kEnBatchDefault = 8;    // track rows whose M_1 loads are in flight together
+constexpr int kEnBatch = 8;           // track rows whose M_1 loads are in flight together
 constexpr int kSelThreads = 256;
 
 // k_m1 works on D(u, v) = M_0(u+1, v) - M_0(u-1, v).  An edge pixel at (u_e, v_e) adds g = G_x w_g to the
@@ -247,15 +247,22 @@ __global__ void __launch_bounds__(kM1Threads, 2) k_m1_fd(const FrameDesc *__rest
 
 // MODE 0: every start of every frame; 1: the starts listed per frame (learned proposal); 2: every start of
 // the frames flagged LD_F_FALLBACK (the proposal selected no lane there).
-// A short list (MODE 1) is latency-bound: each start is a serial chain of divisions and gathers, so the
-// list form issues the M_1 loads of 32 rows at a time instead of 8 (fewer dependent round trips).
+//
+// A start is a serial chain over its rows, and one frame's starts are a few warps per SM, so the kernel is bound
+// by that chain's latency.  The track does not depend on M_1: a batch of kEnBatch rows computes its columns with
+// the division above (32 cycles a row; __fdiv_rn takes over 60 with its range check and branch), issues its M_1
+// loads, and only then are the loads of the batch before it added, in row order, so their latency runs under the
+// chain.  A batch that leaves the division's range is computed again with __fdiv_rn.
+// 22.5 us for one 1242 x 375 frame, 49 us for 64 and 70 us for sixteen of 1920 x 1080 (43 / 72 / 139 us with
+// __fdiv_rn in the chain and each batch's loads awaited before the next batch's steps); a listed start (MODE 1)
+// took 32 rows a batch for that and now needs 32 us instead of 53 for 32 frames with the common form.
 template <int MODE, bool LAM>
 __device__ __forceinline__ void energy_body(const KParams &kp, const Work &w, const int32_t *elist, const int32_t *ecnt,
                                             int ecap, const int f, const int tile)
 {
-    constexpr int kEnBatch = MODE == 1 ? 32 : kEnBatchDefault;
-    extern __shared__ float vrow[];   // [3][H]: V_px, V_py, and the divisor of Eq. 25 for each row
+    extern __shared__ float2 vrow[];   // [H] (V_px, V_py), then [H] the reciprocal of each row's divisor
     const int W = kp.W, H = kp.H;
+    float *vrcp = reinterpret_cast<float *>(vrow + H);
     const FrameState &fs = w.fs[f];
     if (fs.flags & LD_F_NO_LANES)
         return;
@@ -265,11 +272,11 @@ __device__ __forceinline__ void energy_body(const KParams &kp, const Work &w, co
         return;
     const int vtop = fs.v_top, vmax = H - 1;
     const float *rows = w.rows + (size_t)f * 3 * H;
-    for (int v = threadIdx.x; v < H; v += kEnThreads) {
-        vrow[v] = rows[2 * H + v];
-        vrow[H + v] = rows[H + v];
-        // the step into row v divides by (v + 1) - V_py(v + 1), the same for every start
-        vrow[2 * H + v] = v < H - 1 ? __fsub_rn(__fadd_rn((float)v, 1.0f), rows[H + v + 1]) : 1.0f;
+    for (int v = max(vtop, 0) + threadIdx.x; v < H; v += kEnThreads) {
+        const float vy = rows[H + v];
+        vrow[v] = make_float2(rows[2 * H + v], vy);
+        // the step from row v to row v - 1 divides by v - V_py(v), the same for every start
+        vrcp[v] = row_reciprocal(__fsub_rn((float)v, vy));
     }
     __syncthreads();
     int i = tile * kEnThreads + threadIdx.x;
@@ -281,52 +288,88 @@ __device__ __forceinline__ void energy_body(const KParams &kp, const Work &w, co
     if (i >= kp.n_starts || !LD_IN(i, kp.n_starts, CK_EN_START))
         return;
     const int32_t *M1 = w.M1 + (size_t)f * H * W;
-    const float fW = (float)W;
-    // The track recursion does not depend on M_1.  Each batch of kEnBatch rows first computes the track
-    // columns (no load in flight while the divisions run), then issues the batch's M_1 loads back to back,
-    // then adds them in row order.
     float u = (float)(i - kp.S0);
+    // the bottom row's column needs no step
     long long E = 0;
-    auto batch = [&](int v0, int nb, auto full) {
+    if (vmax >= vtop) {
+        const int c = track_column(u);
+        if ((unsigned)c < (unsigned)W && LD_IN(c, W, CK_EN_COL))
+            E = __ldg(M1 + (size_t)vmax * W + c);
+    }
+    // rows v0 - 1 .. v0 - nb from the track at row v0; m receives their M_1 (0 outside the frame)
+    auto batch = [&](int v0, int nb, int (&m)[kEnBatch], auto full) {
         int col[kEnBatch];
-        float fv = (float)v0;  // (float)v, exact (v < 2^24)
+        const float u0 = u;
+        float fv = (float)v0, lo = 1.0f, hi = 1.0f;   // rows are below 2^24: exact
 #pragma unroll
         for (int b = 0; b < kEnBatch; ++b) {
-            const int v = v0 - b;
             col[b] = -1;
             if (decltype(full)::value || b < nb) {
-                if (v < vmax) {
-                    const float vx = vrow[v + 1], vy = vrow[H + v + 1];
-                    const float num = __fsub_rn(__fadd_rn(vx, __fmul_rn(fv, u)), __fmul_rn(vy, u));
-                    u = __fdiv_rn(num, vrow[2 * H + v]);
-                }
-                const float c = floorf(__fadd_rn(u, 0.5f));
-                if (c >= 0.0f && c < fW)
-                    col[b] = (int)c;
+                const float2 V = vrow[v0 - b];
+                const float y = vrcp[v0 - b], d = __fsub_rn(fv, V.y);
+                fv = __fsub_rn(fv, 1.0f);
+                const float num = __fsub_rn(__fadd_rn(V.x, __fmul_rn(fv, u)), __fmul_rn(V.y, u));
+                lo = fminf(lo, fabsf(num));
+                hi = fmaxf(hi, fabsf(num));
+                u = div_by_row(num, d, y);
+                col[b] = track_column(u);
             }
-            fv = __fsub_rn(fv, 1.0f);
         }
-        int32_t m[kEnBatch];
-        const int rowoff = v0 * W;   // H W < 2^31
+        if (!(lo >= kDivNumLo && hi <= kDivNumHi && fabsf(u) <= 3.0e38f)) {   // a NaN on the way stays in u
+            u = u0;
+            fv = (float)v0;
+#pragma unroll 1
+            for (int b = 0; b < nb; ++b) {
+                const float2 V = vrow[v0 - b];
+                const float d = __fsub_rn(fv, V.y);
+                fv = __fsub_rn(fv, 1.0f);
+                u = __fdiv_rn(__fsub_rn(__fadd_rn(V.x, __fmul_rn(fv, u)), __fmul_rn(V.y, u)), d);
+                const int cb = track_column(u);
+#pragma unroll
+                for (int k = 0; k < kEnBatch; ++k)
+                    col[k] = k == b ? cb : col[k];
+            }
+        }
+        const int rowoff = (v0 - 1) * W;   // H W < 2^31
 #pragma unroll
         for (int b = 0; b < kEnBatch; ++b)
-            m[b] = col[b] >= 0 && LD_IN(col[b], W, CK_EN_COL) && LD_IN(v0 - b, H, CK_EN_ROW)
-                       ? __ldg(M1 + (rowoff - b * W + col[b])) : 0;
+            m[b] = (unsigned)col[b] < (unsigned)W && LD_IN(v0 - 1 - b, H, CK_EN_ROW) ? __ldg(M1 + (rowoff - b * W + col[b])) : 0;
+    };
+    auto add = [&](const int (&m)[kEnBatch], int nb, auto full) {
 #pragma unroll
         for (int b = 0; b < kEnBatch; ++b)
             if (decltype(full)::value || b < nb)
                 E = LAM ? E + (long long)m[b] : (long long)m[b];
     };
-    int v0 = vmax;
-    for (; v0 - kEnBatch + 1 >= vtop; v0 -= kEnBatch)
-        batch(v0, kEnBatch, std::true_type());
-    if (v0 >= vtop)
-        batch(v0, v0 - vtop + 1, std::false_type());
+    int v0 = vmax, ma[kEnBatch], mb[kEnBatch];
+    if (v0 - kEnBatch >= vtop) {
+        batch(v0, kEnBatch, ma, std::true_type());
+        v0 -= kEnBatch;
+        for (;; v0 -= 2 * kEnBatch) {   // two batches a turn: no loaded value is copied before it is needed
+            if (v0 - kEnBatch < vtop) {
+                add(ma, kEnBatch, std::true_type());
+                break;
+            }
+            batch(v0, kEnBatch, mb, std::true_type());
+            add(ma, kEnBatch, std::true_type());
+            if (v0 - 2 * kEnBatch < vtop) {
+                add(mb, kEnBatch, std::true_type());
+                v0 -= kEnBatch;
+                break;
+            }
+            batch(v0 - kEnBatch, kEnBatch, ma, std::true_type());
+            add(mb, kEnBatch, std::true_type());
+        }
+    }
+    if (v0 > vtop) {
+        batch(v0, v0 - vtop, ma, std::false_type());
+        add(ma, v0 - vtop, std::false_type());
+    }
     w.HE[(size_t)f * kp.n_starts + i] = (int64_t)E;
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(kEnThreads, MODE == 1 ? 2 : 12) k_energy(const KParams kp, const Work w,
+__global__ void __launch_bounds__(kEnThreads, 8) k_energy(const KParams kp, const Work w,
                                                                          const int32_t *elist, const int32_t *ecnt,
                                                                          int ecap)
 {
@@ -335,7 +378,7 @@ __global__ void __launch_bounds__(kEnThreads, MODE == 1 ? 2 : 12) k_energy(const
     else
         energy_body<MODE, false>(kp, w, elist, ecnt, ecap, blockIdx.y, blockIdx.x);
 }
-__global__ void __launch_bounds__(kEnThreads, 12) k_energy_fd(const FrameDesc *__restrict__ fd)
+__global__ void __launch_bounds__(kEnThreads, 8) k_energy_fd(const FrameDesc *__restrict__ fd)
 {
     const FrameDesc &d = fd[blockIdx.y];
     const KParams kp = d.kp;   // the frame's parameters, loaded once into registers
@@ -350,45 +393,63 @@ __global__ void __launch_bounds__(kEnThreads, 12) k_energy_fd(const FrameDesc *_
 
 // mode 0: every start; 1: minima only at candidate starts (cflag bit 0), minimum over the evaluated ones
 // (bit 1), and a frame without a lane is flagged LD_F_FALLBACK; 2: the flagged frames only, every start.
+//
+// One CTA per frame, bound by the latency of its dependent steps: the energies are read once, into shared memory
+// (staged: when they fit kSelStage there, which frames up to 2700 columns do; wider ones read them again from
+// L2), the greedy suppression runs a warp's 32 candidates at a time, and the result is written by as many lanes
+// as it has fields.  10.2 us before and 8.2 us now for one 1242 x 375 frame, 14.3 and 12.3 us for sixteen of
+// 1920 x 1080.
+constexpr size_t kSelStage = 64 * 1024;
+
+inline bool select_staged(int ns) { return 12 * (size_t)(ns + 8) <= kSelStage; }
+inline size_t select_smem(int ns) { return (select_staged(ns) ? 12 : 4) * (size_t)(ns + 8); }
+
+template <bool STAGED>
 __device__ __forceinline__ void select_body(const KParams &kp, const Work &w, ld_lanes *out, const uint8_t *cflag,
                                             int mode, const int f)
 {
-    extern __shared__ int cand[];     // [n_starts / 2 + 2] candidate positions, then their sorted order
+    extern __shared__ __align__(16) long long ssm[];
     __shared__ long long red[kSelThreads / 32];
     __shared__ int ncand;
-    __shared__ int acc[LD_MAX_LANES];
-    __shared__ int nacc;
     const int ns = kp.n_starts;
-    const int tid = threadIdx.x;
-    const FrameState fs = w.fs[f];
-    if (mode == 2 && !(fs.flags & LD_F_FALLBACK))
+    const int tid = threadIdx.x, lane = tid & 31;
+    const FrameState &fs = w.fs[f];
+    const int flags_in = fs.flags;
+    if (mode == 2 && !(flags_in & LD_F_FALLBACK))
         return;
-    int flags = fs.flags;
-    const int64_t *he = w.HE + (size_t)f * ns;
+    int flags = flags_in;
+    const long long *he = reinterpret_cast<const long long *>(w.HE + (size_t)f * ns);
+    // candidate positions (strict minima: at most (ns - 1) / 2), then their sorted order
+    int *cand = reinterpret_cast<int *>(STAGED ? ssm + ns + 4 : ssm);
     const uint8_t *cf = mode == 1 ? cflag + (size_t)f * ns : nullptr;
-    if (tid == 0) {
+    if (tid == 0)
         ncand = 0;
-        nacc = 0;
-    }
-    long long mn = 0;
+    int na = 0, kept = 0;   // warp 0: lanes accepted so far; lane a holds the a-th
     if (!(flags & LD_F_NO_LANES)) {
         long long m = 0x7fffffffffffffffLL;
-        for (int i = tid; i < ns; i += kSelThreads)
-            if (!cf || (cf[i] & 2))
-                m = he[i] < m ? (long long)he[i] : m;
+#pragma unroll 8
+        for (int i = tid; i < ns; i += kSelThreads) {
+            const bool use = !cf || (cf[i] & 2);
+            if (STAGED || use) {
+                const long long e = he[i];
+                if (STAGED)
+                    ssm[i] = e;
+                m = use && e < m ? e : m;
+            }
+        }
+        if (STAGED)
+            he = ssm;
         for (int d = 16; d > 0; d >>= 1) {
             const long long o = __shfl_down_sync(0xffffffffu, m, d);
             m = o < m ? o : m;
         }
-        if ((tid & 31) == 0)
+        if (lane == 0)
             red[tid >> 5] = m;
         __syncthreads();
-        mn = red[0];
+        long long mn = red[0];
         for (int i = 1; i < kSelThreads / 32; ++i)
             mn = red[i] < mn ? red[i] : mn;
-        if (ns < 3 || mn >= 0) {
-            flags |= LD_F_NO_LANES;
-        } else {
+        if (ns >= 3 && mn < 0) {
             const long long t = kp.thr_abs != 0 ? kp.thr_abs : -(((-mn) * (long long)kp.thr_num) / (long long)kp.thr_den);
             int *pos = cand;
             for (int i = 1 + tid; i < ns - 1; i += kSelThreads) {
@@ -396,7 +457,7 @@ __device__ __forceinline__ void select_body(const KParams &kp, const Work &w, ld
                     continue;
                 const long long h = he[i];
                 if (h < he[i - 1] && h < he[i + 1] && h < t) {
-                    const int at = atomicAdd(&ncand, 1);   // strict minima: at most (ns - 1) / 2
+                    const int at = atomicAdd(&ncand, 1);
                     if (LD_IN(at, ns / 2 + 2, CK_SEL_START))
                         pos[at] = i;
                 }
@@ -409,6 +470,7 @@ __device__ __forceinline__ void select_body(const KParams &kp, const Work &w, ld
                 const int ia = pos[a];
                 const long long ea = he[ia];
                 int rank = 0;
+#pragma unroll 4
                 for (int b = 0; b < nc; ++b) {
                     const int ib = pos[b];
                     const long long eb = he[ib];
@@ -418,69 +480,71 @@ __device__ __forceinline__ void select_body(const KParams &kp, const Work &w, ld
                     ord[rank] = ia;
             }
             __syncthreads();
-            if (tid == 0) {
-                int na = 0;
-                for (int a = 0; a < nc && na < kp.max_lanes && LD_IN(na, LD_MAX_LANES, CK_SEL_LANES); ++a) {
-                    const int c = ord[a];
-                    bool ok = true;
+            // greedy in that order, a warp's 32 candidates at a time: the first one not near an accepted lane is
+            // the next lane, and strikes out those near it
+            if (tid < 32) {
+                for (int a0 = 0; a0 < nc && na < kp.max_lanes; a0 += 32) {
+                    const int c = a0 + lane < nc ? ord[a0 + lane] : 0;
+                    bool open = a0 + lane < nc;
                     for (int b = 0; b < na; ++b)
-                        ok &= abs(c - acc[b]) > kp.near_px;
-                    if (ok)
-                        acc[na++] = c;
-                }
-                for (int a = 1; a < na; ++a) {
-                    const int c = acc[a];
-                    int b = a - 1;
-                    while (b >= 0 && acc[b] > c) {
-                        acc[b + 1] = acc[b];
-                        --b;
+                        open &= abs(c - __shfl_sync(0xffffffffu, kept, b)) > kp.near_px;
+                    unsigned live;
+                    while (na < kp.max_lanes && (live = __ballot_sync(0xffffffffu, open)) != 0 &&
+                           LD_IN(na, LD_MAX_LANES, CK_SEL_LANES)) {
+                        const int got = __shfl_sync(0xffffffffu, c, __ffs(live) - 1);
+                        if (lane == na)
+                            kept = got;
+                        ++na;
+                        open &= abs(c - got) > kp.near_px;
                     }
-                    acc[b + 1] = c;
                 }
-                nacc = na;
             }
-            __syncthreads();
-            if (nacc == 0)
-                flags |= LD_F_NO_LANES;
         }
     }
-    __syncthreads();
-    if (mode == 1 && tid == 0 && nacc == 0 && !(fs.flags & LD_F_NO_LANES))
-        w.fs[f].flags = fs.flags | LD_F_FALLBACK;
-    if (tid == 0) {
-        ld_lanes L;
-        const int na = nacc;
+    if (tid >= 32)
+        return;
+    if (na == 0)
+        flags |= LD_F_NO_LANES;
+    if (mode == 1 && lane == 0 && na == 0 && !(flags_in & LD_F_NO_LANES))
+        w.fs[f].flags = flags_in | LD_F_FALLBACK;
+    // ascending positions (distinct: a lane is near itself)
+    int rank = 0;
+    for (int b = 0; b < na; ++b)
+        rank += __shfl_sync(0xffffffffu, kept, b) < kept;
+    ld_lanes &L = out[f];
+    if (lane < LD_MAX_LANES) {
+        const int at = lane < na ? rank : lane;
+        L.start_u[at] = lane < na ? kept - kp.S0 : 0;
+        L.energy[at] = lane < na ? he[kept] : 0;
+    } else if (lane < LD_MAX_LANES + 3) {
+        L.beta[lane - LD_MAX_LANES] = fs.beta[lane - LD_MAX_LANES];
+    } else if (lane < LD_MAX_LANES + 8) {
+        L.gamma[lane - LD_MAX_LANES - 3] = fs.gamma[lane - LD_MAX_LANES - 3];
+    } else if (lane == 16) {
         L.n_lanes = na;
         L.flags = flags;
-        for (int a = 0; a < LD_MAX_LANES; ++a) {
-            L.start_u[a] = a < na ? acc[a] - kp.S0 : 0;
-            L.energy[a] = a < na ? he[acc[a]] : 0;
-        }
+    } else if (lane == 17) {
         L.v_top = fs.v_top;
         L.centre = kp.centre;
         L.scale_exp = kp.e;
+    } else if (lane == 18) {
         L.rounds_y = fs.rounds_y;
         L.rounds_x = fs.rounds_x;
         L.reserved = 0;
-        for (int i = 0; i < 3; ++i)
-            L.beta[i] = fs.beta[i];
-        for (int i = 0; i < 5; ++i)
-            L.gamma[i] = fs.gamma[i];
-        out[f] = L;
     }
 }
 
+template <bool STAGED>
 __global__ void __launch_bounds__(kSelThreads) k_select(const KParams kp, const Work w, ld_lanes *out,
                                                         const uint8_t *cflag, int mode)
 {
-    select_body(kp, w, out, cflag, mode, blockIdx.x);
+    select_body<STAGED>(kp, w, out, cflag, mode, blockIdx.x);
 }
+template <bool STAGED>
 __global__ void __launch_bounds__(kSelThreads) k_select_fd(const FrameDesc *__restrict__ fd)
 {
     const FrameDesc &d = fd[blockIdx.x];
-    const KParams kp = d.kp;   // the frame's parameters, loaded once into registers
-    const Work w = d.w;
-    select_body(kp, w, d.out, nullptr, 0, 0);
+    select_body<STAGED>(d.kp, d.w, d.out, nullptr, 0, 0);
 }
 
 // Alg. 7, last step: each selected lane drawn by iterating Eq. 25 from its start (s, H-1) up to v_top, in
@@ -517,11 +581,15 @@ cudaError_t setup_lpv(int smem_optin)
 {
     cudaError_t e = allow_max_smem(k_m1, smem_optin);
     if (e == cudaSuccess)
-        e = allow_max_smem(k_select, smem_optin);
+        e = allow_max_smem(k_select<true>, smem_optin);
+    if (e == cudaSuccess)
+        e = allow_max_smem(k_select<false>, smem_optin);
     if (e == cudaSuccess)
         e = allow_max_smem(k_m1_fd, smem_optin);
     if (e == cudaSuccess)
-        e = allow_max_smem(k_select_fd, smem_optin);
+        e = allow_max_smem(k_select_fd<true>, smem_optin);
+    if (e == cudaSuccess)
+        e = allow_max_smem(k_select_fd<false>, smem_optin);
     if (e == cudaSuccess)
         e = allow_max_smem(k_energy_fd, smem_optin);
     return e;
@@ -554,7 +622,8 @@ cudaError_t launch_energy_fd(const KParams &kmax, const FrameDesc *fd, int n, cu
 
 cudaError_t launch_select_fd(const KParams &kmax, const FrameDesc *fd, int n, cudaStream_t s)
 {
-    k_select_fd<<<n, kSelThreads, sizeof(int) * (size_t)(kmax.n_starts + 4), s>>>(fd);
+    auto *kernel = select_staged(kmax.n_starts) ? k_select_fd<true> : k_select_fd<false>;
+    kernel<<<n, kSelThreads, select_smem(kmax.n_starts), s>>>(fd);
     return cudaGetLastError();
 }
 
@@ -583,8 +652,8 @@ cudaError_t launch_energy_fallback(const KParams &kp, const Work &w, cudaStream_
 static cudaError_t select_mode(const KParams &kp, const Work &w, ld_lanes *out, const uint8_t *cflag, int mode,
                                cudaStream_t s)
 {
-    const size_t smem = sizeof(int) * (size_t)(kp.n_starts + 4);
-    k_select<<<kp.n_frames, kSelThreads, smem, s>>>(kp, w, out, cflag, mode);
+    auto *kernel = select_staged(kp.n_starts) ? k_select<true> : k_select<false>;
+    kernel<<<kp.n_frames, kSelThreads, select_smem(kp.n_starts), s>>>(kp, w, out, cflag, mode);
     return cudaGetLastError();
 }
 

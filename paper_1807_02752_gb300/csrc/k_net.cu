@@ -1204,31 +1204,63 @@ __global__ void k_labels(const KParams kp, const Work w, const ld_lanes *lanes, 
     }
 }
 
-// one thread per (frame, coarse start c): the heatmap summed along the track in steps of four rows
-__global__ void __launch_bounds__(128) k_score(const KParams kp, const Work w, const float *z, float *scores,
-                                               int mh, int mw)
+// one thread per (frame, coarse start c): the heatmap summed along the track in steps of four rows.  Bound by the
+// chain of its steps: the rows' reciprocals are formed once per CTA, and a batch of eight steps is taken before
+// the heatmap values of the one before it are added (in row order; a step outside the frame adds 0, which a
+// running sum that starts at +0 ignores).  12.6 us for 32 frames of 1242 x 375, 31 us with a division and a
+// dependent addition per step.
+constexpr int kScThreads = 128, kScBatch = 8;
+
+__global__ void __launch_bounds__(kScThreads) k_score(const KParams kp, const Work w, const float *z, float *scores,
+                                                      int mh, int mw)
 {
-    const int f = blockIdx.y, c = blockIdx.x * 128 + threadIdx.x;
+    extern __shared__ float srow[];   // [steps] V_px, V_py, reciprocal of v - V_py, for v = H - 1, H - 5, ...
+    const int f = blockIdx.y, c = blockIdx.x * kScThreads + threadIdx.x;
     const int nc = (kp.n_starts + 3) >> 2;
-    if (c >= nc)
-        return;
     const FrameState &fs = w.fs[f];
     float acc = 0.0f;
     if (!(fs.flags & LD_F_NO_LANES)) {
-        const int W = kp.W, H = kp.H;
+        const int W = kp.W, H = kp.H, vtop = fs.v_top;
+        const int steps = vtop < H ? (H - 1 - vtop) / 4 + 1 : 0;
         const float *Vpy = w.rows + (size_t)f * 3 * H + H;
         const float *Vpx = Vpy + H;
         const float *zf = z + (size_t)f * mh * mw;
-        float u = __fadd_rn((float)(4 * c - kp.S0), 1.5f);
-        for (int v = H - 1; v >= fs.v_top; v -= 4) {
-            const float col = floorf(__fadd_rn(u, 0.5f));
-            if (col >= 0.0f && col < (float)W)
-                acc = __fadd_rn(acc, __ldg(zf + (v >> 2) * mw + ((int)col >> 2)));
-            const float step = __fdiv_rn(__fmul_rn(4.0f, __fsub_rn(Vpx[v], u)), __fsub_rn((float)v, Vpy[v]));
-            u = __fadd_rn(u, step);
+        for (int k = threadIdx.x; k < steps; k += kScThreads) {
+            const int v = H - 1 - 4 * k;
+            srow[3 * k] = Vpx[v];
+            srow[3 * k + 1] = Vpy[v];
+            srow[3 * k + 2] = row_reciprocal(__fsub_rn((float)v, Vpy[v]));
         }
+        __syncthreads();
+        float u = __fadd_rn((float)(4 * c - kp.S0), 1.5f), val[kScBatch] = {};
+        for (int k0 = 0; k0 < steps; k0 += kScBatch) {
+            int col[kScBatch];
+#pragma unroll
+            for (int b = 0; b < kScBatch; ++b) {
+                const int k = k0 + b;
+                col[b] = -1;
+                if (k < steps) {
+                    col[b] = track_column(u);
+                    const float vx = srow[3 * k], vy = srow[3 * k + 1], y = srow[3 * k + 2];
+                    const float num = __fmul_rn(4.0f, __fsub_rn(vx, u)), d = __fsub_rn((float)(H - 1 - 4 * k), vy);
+                    float q = div_by_row(num, d, y);
+                    if (!(fabsf(num) >= kDivNumLo && fabsf(num) <= kDivNumHi && y == y))
+                        q = __fdiv_rn(num, d);
+                    u = __fadd_rn(u, q);
+                }
+            }
+#pragma unroll
+            for (int b = 0; b < kScBatch; ++b) {
+                acc = __fadd_rn(acc, val[b]);
+                val[b] = (unsigned)col[b] < (unsigned)W ? __ldg(zf + ((H - 1 - 4 * (k0 + b)) >> 2) * mw + (col[b] >> 2)) : 0.0f;
+            }
+        }
+#pragma unroll
+        for (int b = 0; b < kScBatch; ++b)
+            acc = __fadd_rn(acc, val[b]);
     }
-    scores[(size_t)f * nc + c] = acc;
+    if (c < nc)
+        scores[(size_t)f * nc + c] = acc;
 }
 
 // one CTA per frame: the top_k coarse scores (ties to the smaller index), flags of candidate (bit 0) and
@@ -1611,8 +1643,8 @@ cudaError_t net_propose(const KParams &kp, const Work &w, const float *z, int mh
                         uint8_t *cflag, int32_t *elist, int32_t *ecnt, int ecap, cudaStream_t s)
 {
     const int nc = (kp.n_starts + 3) >> 2;
-    dim3 g1((nc + 127) / 128, kp.n_frames);
-    k_score<<<g1, 128, 0, s>>>(kp, w, z, scores, mh, mw);
+    dim3 g1((nc + kScThreads - 1) / kScThreads, kp.n_frames);
+    k_score<<<g1, kScThreads, sizeof(float) * 3 * (size_t)((kp.H + 3) / 4), s>>>(kp, w, z, scores, mh, mw);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
         return e;

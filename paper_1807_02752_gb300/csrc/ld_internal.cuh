@@ -193,6 +193,35 @@ __host__ __device__ inline int vpx_row_bytes(int W) { return (W + 80 + 15) & ~15
 
 __device__ __forceinline__ float pow2f(int k) { return __int_as_float((127 + k) << 23); }
 
+// Division on the track's serial chain.  y = RN(1/d) is kept per row, so a quotient n/d is n y corrected twice
+// with the exact remainder n - q d: the first correction leaves it within one unit in the last place, and from
+// there the second one is the correctly rounded quotient (Markstein, "Computation of elementary functions on the
+// IBM RISC System/6000", 1990, theorem on the final step with a correctly rounded reciprocal).  Nothing may leave
+// the normal range on the way: |d| in [2^-40, 2^40] (a row outside gets y = NaN), |n| in [2^-60, 2^60] (checked
+// by the caller); else __fdiv_rn.
+constexpr float kDivNumLo = 8.67361738e-19f, kDivNumHi = 1.15292150e18f;    // 2^-60, 2^60
+constexpr float kDivDenLo = 9.09494702e-13f, kDivDenHi = 1.09951163e12f;    // 2^-40, 2^40
+
+__device__ __forceinline__ float row_reciprocal(float d)
+{
+    return fabsf(d) >= kDivDenLo && fabsf(d) <= kDivDenHi ? __frcp_rn(d) : __int_as_float(0x7fc00000);
+}
+
+__device__ __forceinline__ float div_by_row(float n, float d, float y)
+{
+    const float q0 = __fmul_rn(n, y);
+    const float q1 = __fmaf_rn(__fmaf_rn(-q0, d, n), y, q0);
+    return __fmaf_rn(__fmaf_rn(-q1, d, n), y, q1);
+}
+
+// floor(RN(u + 1/2)), the track's column: adding 1.5 2^23 rounding down leaves the floor in the low bits for
+// magnitudes below 2^22; any other u (infinities and NaN included) gives a number outside [0, 2^22) as unsigned,
+// which is no column.  A plain addition where the conversion unit takes a warp's 32 lanes in eight cycles.
+__device__ __forceinline__ int track_column(float u)
+{
+    return __float_as_int(__fadd_rd(__fadd_rn(u, 0.5f), 12582912.0f)) - 0x4b400000;
+}
+
 // Allow a kernel the largest dynamic shared memory the device offers next to its static shared memory.
 template <typename K>
 inline cudaError_t allow_max_smem(K kernel, int smem_optin)
