@@ -40,7 +40,7 @@
 // floor(u + (v - V_py(v)) G_y / G_x + 0.5) in float32 (the line through the pixel perpendicular to the
 // gradient meets row V_py there), kept when inside [0, W).  Edge pixels and votes are appended to per-row
 // lists through one global atomic per row and tile (order within a row is arbitrary; every consumer sums
-// over them); the per-row counts are zeroed before the launch.
+// over them); k_vdisp zeroes the per-row counts.
 #include "ld_internal.cuh"
 
 namespace ld {
@@ -200,7 +200,7 @@ __device__ __forceinline__ void grad_body(const KParams &kp, const Work &w, cons
     const FrameState &fs = w.fs[f];
     const int vtop = fs.v_top;
     if ((fs.flags & LD_F_NO_LANES) || r0 + nr - 1 < vtop)
-        return;   // no road pixel of the tile (the per-row counts were zeroed before the launch)
+        return;   // no road pixel of the tile (k_vdisp zeroed the per-row counts)
     if (!LD_IN(kp.n_cls, kClsTables + 1, CK_GRAD_TILE))   // the class tables the tile copies
         return;
     const GradTile T = grad_tile<RHO>(nr, nj, kp.n_cls);

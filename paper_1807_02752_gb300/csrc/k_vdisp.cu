@@ -53,9 +53,11 @@ __device__ __forceinline__ float4 ld_stream(const float4 *p, uint64_t pol)
     return v;
 }
 
-// Rows [tile * kRows, ..) of frame f.
-__device__ __forceinline__ void vdisp_body(const KParams &kp, int32_t *__restrict__ myT, const float *__restrict__ disp,
-                                           int kRows, int f, int tile)
+// Rows [tile * kRows, ..) of frame f.  Their edge and vote counts, to which the gradient kernel's tiles append later
+// in the sequence, are zeroed here: as two fills of their own they cost a one-frame call about 4 us of launches.
+__device__ __forceinline__ void vdisp_body(const KParams &kp, int32_t *__restrict__ myT, int32_t *__restrict__ ecount,
+                                           int32_t *__restrict__ vcount, const float *__restrict__ disp, int kRows, int f,
+                                           int tile)
 {
     extern __shared__ int32_t hist[];  // [kRows][D + 1]
     const int W = kp.W, H = kp.H, D = kp.D, Dp = D + 1;
@@ -64,6 +66,10 @@ __device__ __forceinline__ void vdisp_body(const KParams &kp, int32_t *__restric
     const int tid = threadIdx.x;
     for (int i = tid; i < kRows * Dp; i += kThreads)
         hist[i] = 0;
+    if (tid < nr) {   // at most one row per thread (vdisp_rows)
+        ecount[(size_t)f * H + r0 + tid] = 0;
+        vcount[(size_t)f * H + r0 + tid] = 0;
+    }
     __syncthreads();
 
     const float *src = disp + ((size_t)f * H + r0) * W;
@@ -147,9 +153,10 @@ __device__ __forceinline__ void vdisp_body(const KParams &kp, int32_t *__restric
 }
 
 __global__ void __launch_bounds__(kThreads) k_vdisp(const KParams kp, int32_t *__restrict__ myT,
+                                                    int32_t *__restrict__ ecount, int32_t *__restrict__ vcount,
                                                     const float *__restrict__ disp, int kRows)
 {
-    vdisp_body(kp, myT, disp, kRows, blockIdx.y, blockIdx.x);
+    vdisp_body(kp, myT, ecount, vcount, disp, kRows, blockIdx.y, blockIdx.x);
 }
 
 __global__ void __launch_bounds__(kThreads) k_vdisp_fd(const FrameDesc *__restrict__ fd, int kRows)
@@ -159,7 +166,7 @@ __global__ void __launch_bounds__(kThreads) k_vdisp_fd(const FrameDesc *__restri
     const Work w = d.w;
     if ((int)blockIdx.x * kRows >= kp.H)
         return;
-    vdisp_body(kp, w.myT, d.disp, kRows, 0, blockIdx.x);
+    vdisp_body(kp, w.myT, w.ecount, w.vcount, d.disp, kRows, 0, blockIdx.x);
 }
 }  // namespace
 
@@ -178,7 +185,7 @@ cudaError_t launch_vdisp(const KParams &kp, const Work &w, const float *disp, cu
     const int kRows = vdisp_rows(kp);
     dim3 grid((kp.H + kRows - 1) / kRows, kp.n_frames);
     const size_t smem = sizeof(int32_t) * kRows * (kp.D + 1);
-    k_vdisp<<<grid, kThreads, smem, s>>>(kp, w.myT, disp, kRows);
+    k_vdisp<<<grid, kThreads, smem, s>>>(kp, w.myT, w.ecount, w.vcount, disp, kRows);
     return cudaGetLastError();
 }
 

@@ -320,15 +320,12 @@ int enqueue_range(ld_handle *h, const ld::KParams &kp, const ld::Work &w, const 
     cudaError_t e = cudaSuccess;
     const size_t npx = (size_t)kp.n_frames * kp.H * kp.W;
     // buffer resets before stage k: stage capture (I^bf starts at -1, not computed; m_x at 0, rows above
-    // v_top) and the per-row lists the gradient kernel's tiles append their edges and votes to.  No earlier
-    // stage touches these buffers, so the timed form makes them before its first event, which keeps them
-    // out of the per-kernel times.
+    // v_top).  No earlier stage touches these buffers, so the timed form makes them before its first event,
+    // which keeps them out of the per-kernel times.  (The per-row edge and vote counts are zeroed by stage 0:
+    // every range starts there.)
     auto resets = [&](int k) -> int {
         if (k == 3 && w.dbg_ibf && (e = cudaMemsetAsync(w.dbg_ibf, 0xff, npx * 2, s)) != cudaSuccess)
             return cuda_fail(h, e, "capture reset");
-        if (k == 3 && ((e = cudaMemsetAsync(w.ecount, 0, (size_t)kp.n_frames * kp.H * 4, s)) != cudaSuccess ||
-                       (e = cudaMemsetAsync(w.vcount, 0, (size_t)kp.n_frames * kp.H * 4, s)) != cudaSuccess))
-            return cuda_fail(h, e, "edge count reset");
         if (k == 4 && w.dbg_mx && (e = cudaMemsetAsync(w.dbg_mx, 0, npx * 4, s)) != cudaSuccess)
             return cuda_fail(h, e, "capture reset");
         return LD_OK;
@@ -588,7 +585,7 @@ int enqueue_mixed_half(ld_handle *h, const ld::KParams &kl, const ld::FrameDesc 
 }
 
 // The two halves of a mixed call on the handle's sub-streams, forked from and joined back to its stream;
-// the per-row edge counts (and the stage capture) of every frame slot are reset first.
+// the stage capture of every frame slot is reset first.
 int enqueue_mixed(ld_handle *h, const MixedHalf half[2], const ld::FrameDesc *fd, int n)
 {
     cudaStream_t s = h->stream;
@@ -598,9 +595,6 @@ int enqueue_mixed(ld_handle *h, const MixedHalf half[2], const ld::FrameDesc *fd
         return cuda_fail(h, e, "capture reset");
     if (h->w.dbg_mx && (e = cudaMemsetAsync(h->w.dbg_mx, 0, px * 4, s)) != cudaSuccess)
         return cuda_fail(h, e, "capture reset");
-    if ((e = cudaMemsetAsync(h->w.ecount, 0, rows * 4, s)) != cudaSuccess ||
-        (e = cudaMemsetAsync(h->w.vcount, 0, rows * 4, s)) != cudaSuccess)
-        return cuda_fail(h, e, "edge count reset");
     if ((e = cudaEventRecord(h->fork, s)) != cudaSuccess)
         return cuda_fail(h, e, "fork");
     for (int k = 0; k < 2; ++k) {
