@@ -598,8 +598,8 @@ inline SrpShape srp_shape_of(int W, int rho, int dmax, int ctas)
     s.smem = ent + 2 * 4 * (size_t)(s.strips * (S / 2) + 2) + 2 * 4 * kSrpHalo + 6 * 4 * 32 * (size_t)s.strips;
     return s;
 }
-// One CTA per map fills the GPU from about 76 maps on (38 pairs; 2.2 ms as one CTA per map however few the
-// pairs, 0.76 ms for one pair on two clusters of 8); below, a map is split over the largest
+// One CTA per map fills the GPU from about 76 maps on (38 pairs); one pair takes 1.52 ms that way and 0.84 ms on
+// two clusters of 8.  So below that number a map is split over the largest
 // cluster whose CTAs still find an SM each, every one keeping at least 96 pixels.  Frames wider than a CTA's
 // warps hold are always split.
 inline bool srp_fits(const SrpShape &s) { return s.warps <= kSrpMaxWarps && s.prep <= kSrpPrep; }
