@@ -77,9 +77,11 @@ __device__ __forceinline__ uint2 srp_lds2(uint32_t a)
     asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
     return v;
 }
+// Not the .aligned forms: those want a converged warp, and the exchange calls this right after stores that only
+// some lanes make.
 __device__ __forceinline__ void cluster_sync_all()
 {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
 // A lane's two adjacent image columns: the K rows of the block window in K bytes (the newest in byte 0) and
