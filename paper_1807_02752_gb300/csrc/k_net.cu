@@ -1413,8 +1413,10 @@ __global__ void __launch_bounds__(kTopThreads) k_topk(const KParams kp, const Wo
 // ---------------------------------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------------------------------
-// Every kernel here stays under the default 48 KB of dynamic shared memory (k_topk: 2 bytes per start,
-// at most 25 KB for the widest frame), so no opt-in is needed.
+// The convolutions, the weight gradients and the fused forward ask for more than the default 48 KB of dynamic shared
+// memory (k_conv_tc<32, 32> 53 KB, k_wgrad<32, 32> 49 KB, k_net_fused 173 KB).  The opt-in belongs to the
+// current device, so every network makes it for its own (setup_net); the others stay below (k_topk: 2 bytes per start, at
+// most 25 KB for the widest frame).
 
 static int grid_for(int tiles, int per_sm)
 {
@@ -1428,14 +1430,6 @@ template <int CIN, int COUT, int EPI>
 static cudaError_t conv(ConvIO io, cudaStream_t s)
 {
     using S = TcSmem<CIN, COUT>;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_conv_tc<CIN, COUT, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)S::bytes);
-        if (e != cudaSuccess)
-            return e;
-        attr = true;
-    }
     io.tiles_r = (io.mh + kTcRows - 1) / kTcRows;
     io.tiles_c = (io.mw + kTcCols - 1) / kTcCols;
     int *err = nullptr;
@@ -1450,13 +1444,6 @@ static cudaError_t conv(ConvIO io, cudaStream_t s)
 static cudaError_t net_forward_fused(const NetArgs &a, const int32_t *xsum, int n, float *z, bool heat, cudaStream_t s,
                                      const FrameState *road)
 {
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_net_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmem);
-        if (e != cudaSuccess)
-            return e;
-        attr = true;
-    }
     FusedIO io{};
     io.xsum = xsum;
     io.w1 = a.wf[0];
@@ -1480,6 +1467,27 @@ static cudaError_t net_forward_fused(const NetArgs &a, const int32_t *xsum, int 
         return e;
     k_net_fused<<<grid_for(n * io.tiles_r * io.tiles_c, 1), kFusedThreads, kFusedSmem, s>>>(io, err);
     return cudaGetLastError();
+}
+
+// Shared-memory opt-ins of the current device (each always to the same value: networks share the kernels).
+cudaError_t setup_net()
+{
+    cudaError_t e = cudaSuccess;
+    auto allow = [&](auto *kernel, size_t bytes) {
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    allow(k_conv_tc<16, 32, kEpiRelu>, TcSmem<16, 32>::bytes);
+    allow(k_conv_tc<32, 32, kEpiRelu>, TcSmem<32, 32>::bytes);
+    allow(k_conv_tc<32, 16, kEpiHead>, TcSmem<32, 16>::bytes);
+    allow(k_conv_tc<16, 32, kEpiMask>, TcSmem<16, 32>::bytes);
+    allow(k_conv_tc<32, 32, kEpiMask>, TcSmem<32, 32>::bytes);
+    allow(k_conv_tc<32, 16, kEpiMask>, TcSmem<32, 16>::bytes);
+    allow(k_wgrad<32, 16>, WgradShape<32, 16>::bytes);
+    allow(k_wgrad<32, 32>, WgradShape<32, 32>::bytes);
+    allow(k_wgrad<16, 32>, WgradShape<16, 32>::bytes);
+    allow(k_net_fused, kFusedSmem);
+    return e;
 }
 
 cudaError_t net_forward(const NetArgs &a, const int32_t *xsum, int n, float *z, bool keep_a4, bool heat,
@@ -1544,14 +1552,6 @@ static cudaError_t wgrad(const NetArgs &a, const __nv_bfloat16 *dS, const __nv_b
         static_assert(COUT == 16, "k_wgrad1 is the first layer's");
         k_wgrad1<<<G, kConvThreads, 0, s>>>(io);
     } else {
-        static bool attr = false;
-        if (!attr) {
-            cudaError_t e = cudaFuncSetAttribute(k_wgrad<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)WgradShape<CIN, COUT>::bytes);
-            if (e != cudaSuccess)
-                return e;
-            attr = true;
-        }
         k_wgrad<CIN, COUT><<<G, kConvThreads, WgradShape<CIN, COUT>::bytes, s>>>(io);
     }
     cudaError_t e = cudaGetLastError();

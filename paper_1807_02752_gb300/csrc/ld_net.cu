@@ -234,7 +234,9 @@ int ld_net_create(ld_handle *h, int32_t training, ld_net **out)
     a.part = tr ? (float *)(b + o_pt) : nullptr;
     a.part_head = tr ? (float *)(b + o_ph) : nullptr;
     // zero parameters until ld_net_set_params
-    e = cudaMemsetAsync(net->mem, 0, off, ld::handle_stream(h));
+    e = ld::setup_net();
+    if (e == cudaSuccess)
+        e = cudaMemsetAsync(net->mem, 0, off, ld::handle_stream(h));
     if (e == cudaSuccess)
         e = cudaStreamSynchronize(ld::handle_stream(h));
     if (e != cudaSuccess) {

@@ -35,6 +35,8 @@ struct NetArgs {
     int fused = 0;                  // 1: inference forward as one kernel (k_net_fused); 0: one kernel per layer
 };
 
+// shared-memory opt-ins of the network's kernels on the current device
+cudaError_t setup_net();
 // logits (heat = false) or the heatmap sigmoid(z) of every cell; with road (the frames' fit states) only
 // the cells on and just above each frame's road rows (v >= v_top), and nothing for frames without a road
 cudaError_t net_forward(const NetArgs &a, const int32_t *xsum, int n, float *z, bool keep_a4, bool heat,
