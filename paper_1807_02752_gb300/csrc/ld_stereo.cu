@@ -691,10 +691,6 @@ int check_pair(ld_stereo *st, const void *left, const void *right, int w, int hh
 template <int RHO, int NPREP, bool CLUSTER, int WARPS>
 cudaError_t launch_srp_t(const ld::SrpArgs &a, const ld::SrpShape &sh, int n, cudaStream_t s)
 {
-    auto kernel = ld::k_srp<RHO, NPREP, CLUSTER, WARPS>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem);
-    if (e != cudaSuccess)
-        return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(sh.ctas, n, 2);
     cfg.blockDim = dim3(32 * sh.warps);
@@ -707,7 +703,7 @@ cudaError_t launch_srp_t(const ld::SrpArgs &a, const ld::SrpShape &sh, int n, cu
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = CLUSTER ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, a);
+    return cudaLaunchKernelEx(&cfg, ld::k_srp<RHO, NPREP, CLUSTER, WARPS>, a);
 }
 
 template <int RHO>
@@ -724,6 +720,21 @@ cudaError_t launch_srp(ld::SrpArgs a, int n, cudaStream_t s)
         return launch_srp_t<RHO, 1, true, ld::kSrpFewWarps>(a, sh, n, s);
     return sh.prep <= 2 ? launch_srp_t<RHO, 2, true, ld::kSrpMaxWarps>(a, sh, n, s)
                         : launch_srp_t<RHO, ld::kSrpPrep, true, ld::kSrpMaxWarps>(a, sh, n, s);
+}
+
+// The instances launch_srp can choose, allowed all of the device's shared memory once: they are shared by every handle
+// of the device, so an allowance that followed each call's own need could fall below another thread's launch.
+template <int RHO>
+cudaError_t setup_srp(int smem_optin)
+{
+    cudaError_t e = ld::allow_max_smem(ld::k_srp<RHO, 1, false, ld::kSrpMaxWarps>, smem_optin);
+    if (e == cudaSuccess)
+        e = ld::allow_max_smem(ld::k_srp<RHO, 1, true, ld::kSrpFewWarps>, smem_optin);
+    if (e == cudaSuccess)
+        e = ld::allow_max_smem(ld::k_srp<RHO, 2, true, ld::kSrpMaxWarps>, smem_optin);
+    if (e == cudaSuccess)
+        e = ld::allow_max_smem(ld::k_srp<RHO, ld::kSrpPrep, true, ld::kSrpMaxWarps>, smem_optin);
+    return e;
 }
 
 // both maps and the check on the handle's stream; `timed` records an event before SRP, between, after LRC
@@ -788,7 +799,16 @@ int ld_stereo_create(ld_handle *h, const ld_stereo_params *sp, ld_stereo **out)
     if (st->sp.d_max < 0)
         st->sp.d_max = ld::handle_params(h).n_disp - 1;
     ld::handle_dims(h, &st->max_w, &st->max_h, &st->max_n);
-    cudaError_t e = cudaSuccess;
+    int dev = 0, optin = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess)
+        e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess)
+        e = sp->rho == 1 ? setup_srp<1>(optin) : sp->rho == 2 ? setup_srp<2>(optin) : setup_srp<3>(optin);
+    if (e != cudaSuccess) {
+        delete st;
+        return scuda(nullptr, e, "kernel set-up");
+    }
     const size_t px = (size_t)st->max_n * st->max_w * st->max_h;
     if (e == cudaSuccess)
         e = cudaMalloc(&st->mem, px * (2 + 2 + 4) + 512);

@@ -74,3 +74,23 @@ def test_network_calls_on_a_second_device(fake):
         L.ld_net_destroy(net)
         L.ld_destroy(det)
     assert L.fake_launches() > 40 and L.fake_refused() == 0
+
+
+def test_stereo_calls_keep_what_other_handles_need(fake):
+    """The kernel instances are shared by all handles of a device, also by handles on other threads: a call on narrow
+    frames must not lower the allowance that a call on wide ones has made sure of and is about to launch with."""
+    ld, L = fake
+    for rho in (1, 2, 3):
+        sp = ld.StereoParams()
+        L.ld_stereo_params_default(C.byref(sp))
+        sp.rho = rho
+        for w, n in ((1242, 64), (640, 64), (1242, 1), (320, 1), (4096, 2), (64, 80)):
+            h = 24
+            det, st = _detector(ld, L, w, h, n), C.c_void_p()
+            assert L.ld_stereo_create(det, C.byref(sp), C.byref(st)) == ld.OK
+            left, out = np.zeros((n, h, w), np.uint8), np.zeros((n, h, w), np.float32)
+            assert L.ld_stereo_run(st, left.ctypes.data, left.ctypes.data, w, h, n, out.ctypes.data) == ld.OK
+            L.ld_stereo_destroy(st)
+            L.ld_destroy(det)
+    assert L.fake_launches() > 0 and L.fake_refused() == 0
+    assert L.fake_lowered() == 0, L.fake_first_lowered()
