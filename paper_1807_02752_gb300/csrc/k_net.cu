@@ -227,12 +227,14 @@ __device__ __forceinline__ bool tc_wait(uint32_t mbar, uint32_t parity)
     return false;
 }
 
+// (a warp-wide instruction, which callers reach after loops that end per lane: __syncwarp first)
 template <int N>
 __device__ __forceinline__ void tc_load(uint32_t taddr, uint32_t (&r)[N]);
 
 template <>
 __device__ __forceinline__ void tc_load<16>(uint32_t taddr, uint32_t (&r)[16])
 {
+    __syncwarp();
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
                    "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
@@ -243,6 +245,7 @@ __device__ __forceinline__ void tc_load<16>(uint32_t taddr, uint32_t (&r)[16])
 template <>
 __device__ __forceinline__ void tc_load<32>(uint32_t taddr, uint32_t (&r)[32])
 {
+    __syncwarp();
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
                  "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),

@@ -284,7 +284,8 @@ __device__ __forceinline__ int vpx_forward(const VpxArgs &a, const VpxMem &S, co
             for (; z < end; z += kStep)
                 sts4(z, make_int4(0, 0, 0, 0));
         }
-        asm volatile("bar.sync 1, %0;" ::"n"(32 * kProducers) : "memory");
+        // (barrier.sync, not bar.sync, which wants a converged warp: the loops above end per lane)
+        asm volatile("barrier.sync 1, %0;" ::"n"(32 * kProducers) : "memory");
         if (plain) {
 #pragma unroll
             for (int i = 0; i < kLists; ++i) {
