@@ -291,7 +291,6 @@ __device__ __forceinline__ void fit_body(const KParams &kp, const Work &w, const
     const int centre = kp.centre;
     const float sc = pow2f(-kp.e);
     const float tr = stage == 0 ? kp.tr_y : kp.tr_x;
-    const int n = LD_IN(n0, P + 1, CK_FIT_NPTS) ? n0 : 0;
     for (int i = tid; i < H; i += kFitThreads)
         rcp[i] = __fmul_rn(__frcp_rn((float)max(i, 1)), pow2f(kp.e));
     for (int i = tid; i < kp.hyps; i += kFitThreads)
@@ -305,7 +304,8 @@ __device__ __forceinline__ void fit_body(const KParams &kp, const Work &w, const
         pid[j] = gp[2 * P + j];
     }
     if (stage == 1 && (fs0.flags & LD_F_NO_LANES))
-        return;
+        return;   // k_vpx_dp wrote no points
+    const int n = LD_IN(n0, P + 1, CK_FIT_NPTS) ? n0 : 0;
     const int n_inl = stage == 0 ? kp.D : H;
     uint8_t *inl = stage == 0 ? w.inl_y + (size_t)f * n_inl : w.inl_x + (size_t)f * n_inl;
     for (int i = tid; i < n_inl; i += kFitThreads)
