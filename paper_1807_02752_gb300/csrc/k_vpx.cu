@@ -48,9 +48,19 @@ constexpr int kMaxCells = 20;               // cells per lane at most
 constexpr int kMaxRows = 8;                 // rows between two exchanges at most
 constexpr size_t kRingBytes = 160 * 1024;   // band changes of 2 * rows rows
 constexpr int kBlock = 32;                  // rows of a backtrack block
-constexpr uint32_t kHasVotes = 0x10;        // bit of a cell's byte in a backtrack row, beside the rank
-constexpr int kOffKey = 1 << 29;            // key of a column off the frame on the first row (keys stay below)
+constexpr uint32_t kHasVotes = 0x80;        // bit of a cell's byte in a backtrack row, beside the rank: the band key's sign
+constexpr int kOffKey = 1 << 29;            // key of a column off the frame on the first row (others are at most 0)
 constexpr int kOffRow = 16 * 64;            // and what it pays per row
+// Keys fit 32 bits while 16 |E| does.  The number of a frame's votes settles it for almost every frame (each vote is in at
+// most 2 chi + 1 bands), but most of the frames beyond that fit too, since their votes do not lie in one column.  So in
+// those every exchange looks at the keys: above kKeyFloor, the rows up to the next one cannot leave the range.  Once a key
+// is below, keys are held at the floor and the result is dropped.  A row lowers a key by at most 16 varrho m, and a cell's
+// m is at most W times the smaller of H and 2 chi + 1.  ld_create requires varrho (2 chi + 1) W H < 2^30: with
+// H >= 16 kMaxRows, kMaxRows rows lower a key by less than 2^30, and with a smaller H by at most 16 kMaxRows 16 W H, less
+// than 2^30 as well.  Texture all over 64 frames of 1242 x 375, varrho 16, chi 64: the call takes 864 us; 1579 when every
+// frame whose votes could pass 2^25 went to vpx_forward_wide.
+constexpr int kKeyFloor = -((1 << 30) - (1 << 20));
+static_assert(16LL * kMaxRows * kMaxVoteRho * LD_MAX_W * (16 * kMaxRows - 1) <= 1LL << 30, "rows between two looks at the keys");
 
 __device__ __forceinline__ int lds_s8(uint32_t a)
 {
@@ -246,8 +256,9 @@ struct DpRow {
     }
 };
 
-// The forward DP with packed keys.  Returns the first column minimising row vtop to every thread.
-template <int TAU, int C>
+// The forward DP with packed keys.  Returns the first column minimising row vtop to every thread, or -1 when the keys
+// passed kKeyFloor (looked for when LOOK).
+template <int TAU, int C, bool LOOK>
 __device__ __forceinline__ int vpx_forward(const VpxArgs &a, const VpxMem &S, const VpxPlan &P, int f, int vtop, uint8_t *gbt)
 {
     const int W = a.W, vmax = a.H - 1, RB = vpx_row_bytes(W);
@@ -347,6 +358,7 @@ __device__ __forceinline__ int vpx_forward(const VpxArgs &a, const VpxMem &S, co
     }
     __syncthreads();
     const int steps = (vmax - vtop + R - 1) / R;
+    [[maybe_unused]] int low = 0;                     // lowest key at an exchange
     for (int s = 0; s < steps; ++s) {
         const uint32_t box = sa(S.box + (s & 1) * P.warps * 2 * HC);   // [warps][2][HC]
         if (dp) {
@@ -360,7 +372,8 @@ __device__ __forceinline__ int vpx_forward(const VpxArgs &a, const VpxMem &S, co
             D.edges(c);
             // one basic block a row, so that a row's packing and stores overlap its shuffles
             auto rows = [&](auto capture) {
-#pragma unroll 2
+                constexpr int kUnroll = decltype(capture)::value ? 1 : 2;   // (less to compile where time matters less)
+#pragma unroll kUnroll
                 for (int r = 0; r < n; ++r) {
 #pragma unroll
                     for (int x = 0; x < C / 4; ++x) {
@@ -381,16 +394,22 @@ __device__ __forceinline__ int vpx_forward(const VpxArgs &a, const VpxMem &S, co
                     D.edges(c);
                     store(out, best);
                     out -= RB;
-                    if (decltype(capture)::value && own)
+                    if (decltype(capture)::value && own && a.dbg_mx)
                         for (int x = 0; x < C; ++x)
                             if (u0 + x < W)
                                 a.dbg_mx[((size_t)f * a.H + vhi - r) * W + u0 + x] = nb[x] / 16;
                 }
             };
-            if (a.dbg_mx)
+            if (LOOK || a.dbg_mx)
                 rows(std::true_type());
             else
                 rows(std::false_type());
+            if constexpr (LOOK)
+#pragma unroll
+                for (int x = 0; x < C; ++x) {
+                    low = min(low, D.f[x]);
+                    D.f[x] = max(D.f[x], kKeyFloor);
+                }
             if (s + 1 < steps) {
                 // edge cells the neighbours need: a warp's first owned lanes, and its last
                 auto put = [&](int side, int l0) {
@@ -422,6 +441,9 @@ __device__ __forceinline__ int vpx_forward(const VpxArgs &a, const VpxMem &S, co
                 }
         }
     }
+    if constexpr (LOOK)
+        if (__syncthreads_or(low < kKeyFloor))
+            return -1;
     int bv = 0x7fffffff, bi = 0x7fffffff;
     if (own)
 #pragma unroll
@@ -433,8 +455,17 @@ __device__ __forceinline__ int vpx_forward(const VpxArgs &a, const VpxMem &S, co
     return block_argmin(bv, bi, S.sh + kMaxChunks);
 }
 
-// The same for energies too large to pack (beyond 2^25 times varrho or lambda_x of any real frame): plain
-// rows in shared memory, compare-select in tie order, one barrier per phase of a row.
+// A function of its own for the frames that need the look: as a branch in the others' loop it cost them 2 % of the
+// kernel (64 frames of 1242 x 375: 100.4 us, 98.3 without), as an early end of the loop 6 %.
+template <int TAU, int C>
+__device__ __noinline__ int vpx_forward_look(const VpxArgs a, const VpxMem S, const VpxPlan P, int f, int vtop, uint8_t *gbt)
+{
+    return vpx_forward<TAU, C, true>(a, S, P, f, vtop, gbt);
+}
+
+// The same with plain energies, for a frame whose best path gathers more than 2^26 - 2^16 (67 million; 1242 x 375 pixels
+// with the default parameters cannot hold that much, 1920 x 1080 only if two thirds of all pixels vote for the path's
+// columns): rows in shared memory, compare-select in tie order, two barriers a row, after the packed form in vain.
 __device__ __noinline__ int vpx_forward_wide(const VpxArgs a, const VpxMem S, const VpxPlan P, int f,
                                              int vtop, uint8_t *gbt)
 {
@@ -502,7 +533,7 @@ __device__ __forceinline__ void vpx_dp_body(const VpxArgs &a, const VpxPlan &P, 
     const FrameState fs0 = a.fs[f];
     if (fs0.flags & LD_F_NO_LANES)
         return;
-    const int vtop = fs0.v_top, vmax = H - 1, chi = a.chi;
+    const int vtop = fs0.v_top, vmax = H - 1;
     if (!LD_IN(vtop, H, CK_VPX_TILE) || !LD_IN(W - 1, P.warps * P.own, CK_VPX_TILE))
         return;
 
@@ -532,10 +563,10 @@ __device__ __forceinline__ void vpx_dp_body(const VpxArgs &a, const VpxPlan &P, 
     votes = 0;
     for (int k = 0; k < nw; ++k)
         votes += S.sh[k];
-    // each vote enters at most 2 chi + 1 band rows, so |E| <= varrho (2 chi + 1) votes + lambda_x tau_x rows
-    const bool packed = ((double)a.vote_rho * (2.0 * chi + 1.0) * votes + (double)a.lambda_x * a.tau_x * H) * 16.0 <
-                        536870912.0;
-    const int ustar = packed ? vpx_forward<TAU, C>(a, S, P, f, vtop, gbt) : vpx_forward_wide(a, S, P, f, vtop, gbt);
+    const bool look = 16.0 * a.vote_rho * (2.0 * a.chi + 1.0) * votes >= 2147483648.0 - 1048576.0;
+    int ustar = look ? vpx_forward_look<TAU, C>(a, S, P, f, vtop, gbt) : vpx_forward<TAU, C, false>(a, S, P, f, vtop, gbt);
+    if (ustar < 0)
+        ustar = vpx_forward_wide(a, S, P, f, vtop, gbt);
 
     // ---- backtrack from (ustar, vtop): blocks of kBlock rows.  While lane 0 of warp 0 walks a block, the other
     // warps fetch the columns the next one can reach (2 kBlock rows of tau_x from the current column) and turn

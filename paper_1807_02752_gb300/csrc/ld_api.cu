@@ -212,7 +212,7 @@ const char *check_params(const ld_params *p)
         return "sigma_s, sigma_r, sigma_g must be > 0";
     if (p->edge_thresh < 0 || p->edge_thresh > 4 * 255 * 2)
         return "edge_thresh must be in [0, 2040]";
-    if (p->vote_rho < 1 || p->vote_rho > 16)
+    if (p->vote_rho < 1 || p->vote_rho > ld::kMaxVoteRho)
         return "vote_rho must be in [1, 16]";
     if (p->chi < 0 || p->chi > 256)
         return "chi must be in [0, 256]";

@@ -15,6 +15,7 @@
 namespace ld {
 
 constexpr int kMaxHyps = 256;
+constexpr int kMaxVoteRho = 16;
 constexpr int kWgEntries = 16385;     // Eq. 23 table: sin(dtheta) in [0, 1/2] in steps of 2^-15
 constexpr int kWrEntries = 768;       // Q15 range weight of dI at index 256 + dI (symmetric; entries >= 512 are 0)
 constexpr int kSentinel = 511;        // image value marking taps outside the frame
