@@ -273,7 +273,8 @@ __device__ __forceinline__ int vpx_forward(const VpxArgs &a, const VpxMem &S, co
         int *half = S.ring + (s & 1) * R * stride;
         constexpr int kLists = 2 * kMaxRows / kProducers;
         int src[kLists], col[kLists][2];
-        const bool plain = !a.band_literal;
+        // the literal bottom band has other lists, but only on the rows down to vmax - chi - 1
+        const bool plain = !a.band_literal || v0 < vmax - a.chi - 1;
 #pragma unroll
         for (int i = 0; i < kLists; ++i) {
             const int l = warp - P.warps + i * kProducers, v = v0 - (l >> 1);
