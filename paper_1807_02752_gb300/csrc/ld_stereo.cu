@@ -137,52 +137,135 @@ __device__ __forceinline__ void srp_block_sums(const int *c0, const int *c1, int
         p0[k] = p1[k] + c0[k] - last[k];
 }
 
-// N and D_B of the blocks of A around (u, v) and of B around (ub, v), from the images.
-template <int RHO>
-__device__ void srp_block_nd(const uint8_t *A, const uint8_t *B, int W, int v, int u, int ub, long long &N, long long &D)
-{
-    constexpr int NB = (2 * RHO + 1) * (2 * RHO + 1);
-    int P = 0, sa = 0, sb = 0, Q = 0;
-    for (int y = -RHO; y <= RHO; ++y)
-        for (int x = -RHO; x <= RHO; ++x) {
-            const int g = A[(size_t)(v + y) * W + u + x], h = B[(size_t)(v + y) * W + ub + x];
-            P += g * h;
-            sa += g;
-            sb += h;
-            Q += h * h;
-        }
-    N = NB * P - sa * sb;
-    D = NB * Q - sb * sb;
-}
-
-// The best candidate of pixel (u, v) by exact comparison, for the rare pixel whose two best float scores are
-// too close: candidates are the d <= dhi within t of l0, l1 or l2, ascending; c1 > c2 <=>
-// N1 |N1| D2 > N2 |N2| D1, and c = 0 where a block is constant (then N = 0).
-template <int RHO>
-__device__ __noinline__ int srp_exact_best(const uint8_t *A, const uint8_t *B, int W, int v, int u, int sign, int l0,
-                                           int l1, int l2, int t, int dhi)
-{
-    int best = -1;
-    long long bN = 0, bD = 0;
-    for (int d = max(min(min(l0, l1), l2) - t, 0); d <= min(max(max(l0, l1), l2) + t, dhi); ++d) {
-        if (abs(d - l0) > t && abs(d - l1) > t && abs(d - l2) > t)
-            continue;
-        long long N, D;
-        srp_block_nd<RHO>(A, B, W, v, u, u + sign * d, N, D);
-        bool better = best < 0;
-        if (!better) {
-            if (N == 0 || bN == 0)
-                better = N > bN;
+// Exact comparison, for a pixel whose two best float scores are too close: candidates are the d <= dhi within t of an
+// estimate, ascending, in integers N = n P - s_a s_b and D = n Q - s_b^2 from the columns of the other image that the row's
+// search used; c1 > c2 <=> N1 |N1| D2 > N2 |N2| D1, and c = 0 where a block is constant (then N = 0).  That is one pixel in
+// 10^4 of noise or of a textured pair, but every pixel where an image does not change along its rows or repeats within a
+// search range; two candidates of such a pixel have the same N and D, and nothing is multiplied.  The best one so far:
+struct SrpBest {
+    int d = -1, N = 0, D = 0;
+    __device__ __forceinline__ void consider(int d1, int N1, int D1)
+    {
+        bool better = d < 0;
+        if (!better && (N1 != N || D1 != D)) {
+            if (N1 == 0 || N == 0)
+                better = N1 > N;
             else
-                better = (__int128)(N * (N < 0 ? -N : N)) * bD > (__int128)(bN * (bN < 0 ? -bN : bN)) * D;
+                better = (__int128)((long long)N1 * abs(N1)) * D > (__int128)((long long)N * abs(N)) * D1;
         }
         if (better) {
-            best = d;
-            bN = N;
-            bD = D;
+            d = d1;
+            N = N1;
+            D = D1;
         }
     }
-    return best;
+};
+
+// N and D of the block whose columns are (alo, ahi), of sum sa, in image A and the entries from e on in image B.
+template <int RHO>
+__device__ __forceinline__ void srp_block_nd(const uint32_t *alo, const uint32_t *ahi, int sa, uint32_t buf, uint32_t odd, int e,
+                                             int &N, int &D)
+{
+    constexpr int K = 2 * RHO + 1, NB = K * K;
+    const uint32_t at = buf + 16u * (uint32_t)(e >> 1);
+    const uint32_t ev = at + ((e & 1) ? odd : 0u), od = at + ((e & 1) ? 16u : odd);
+    const uint4 first = srp_lds(ev);
+    unsigned P = __dp4a(alo[0], first.x, __dp4a(ahi[0], first.y, 0u));
+    unsigned Q = __dp4a(first.x, first.x, __dp4a(first.y, first.y, 0u));
+#pragma unroll
+    for (int k = 1; k < K; ++k) {
+        const uint2 b = srp_lds2((k & 1) ? od + 16u * (uint32_t)(k >> 1) : ev + 16u * (uint32_t)(k >> 1));
+        P = __dp4a(alo[k], b.x, __dp4a(ahi[k], b.y, P));
+        Q = __dp4a(b.x, b.x, __dp4a(b.y, b.y, Q));
+    }
+    const int sb = (int)first.z;
+    N = NB * (int)P - sa * sb;
+    D = NB * (int)Q - sb * sb;
+}
+
+// The exact best of pixel (u, v) with the estimates l0, l1, l2, by one lane of a cluster's CTA: the block of A from the
+// image, and where the entries lie (k_srp's layout) worked out again, so that k_srp keeps nothing for it.  One pair of
+// 1242 x 375 that is constant along its rows: 0.95 ms (1.76 with the blocks of both images summed for each candidate).
+template <int RHO>
+__device__ __noinline__ int srp_exact_best(const SrpArgs &a, int v, int u, int l0, int l1, int l2, int t, int dhi)
+{
+    extern __shared__ __align__(16) unsigned char sm[];
+    const int W = a.W, dir = blockIdx.z, rank = blockIdx.x, sign = dir == 0 ? -1 : 1, S = srp_strip(RHO);
+    const uint8_t *block = (dir == 0 ? a.left : a.right) + ((size_t)blockIdx.y * a.H + v - RHO) * W + u - RHO;
+    const int col0 = rank * a.per - (rank > 0 ? kSrpHalo : 0), ent0 = col0 - (dir == 0 ? S * a.n_extra : 0);
+    const uint32_t odd = 16u * (uint32_t)(srp_entries(a.strips, a.n_extra, RHO) >> 1);
+    const uint32_t buf = (uint32_t)__cvta_generic_to_shared(sm) + (uint32_t)(v & 1) * 2u * odd;
+    const int e0 = u - RHO - ent0;
+    constexpr int K = 2 * RHO + 1;
+    uint32_t lo[K], hi[K];   // the block's columns, the top row in byte 0
+    unsigned sa = 0;
+#pragma unroll
+    for (int x = 0; x < K; ++x) {
+        lo[x] = hi[x] = 0u;
+#pragma unroll
+        for (int y = 0; y < K; ++y)
+            (y < 4 ? lo : hi)[x] |= (uint32_t)__ldg(block + (size_t)y * W + x) << (8 * (y & 3));
+        sa = __dp4a(lo[x], 0x01010101u, __dp4a(hi[x], 0x01010101u, sa));
+    }
+    SrpBest best;
+    for (int d = max(min(min(l0, l1), l2) - t, 0); d <= min(max(max(l0, l1), l2) + t, dhi); ++d)
+        if (abs(d - l0) <= t || abs(d - l1) <= t || abs(d - l2) <= t) {
+            int N, D;
+            srp_block_nd<RHO>(lo, hi, (int)sa, buf, odd, e0 + sign * d, N, D);
+            best.consider(d, N, D);
+        }
+    return best.d;
+}
+
+// The lane's two columns and its right neighbours': the K + 1 columns of the blocks of a lane's two pixels.
+template <int RHO>
+__device__ __forceinline__ void srp_columns(const uint32_t (&lo)[2], const uint32_t (&hi)[2], uint32_t (&clo)[2 * RHO + 2],
+                                            uint32_t (&chi)[2 * RHO + 2])
+{
+#pragma unroll
+    for (int x = 0; x <= RHO; ++x)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            clo[2 * x + c] = __shfl_down_sync(0xffffffffu, lo[c], x);
+            chi[2 * x + c] = __shfl_down_sync(0xffffffffu, hi[c], x);
+        }
+}
+
+// What a warp's exact comparison needs of a row.
+struct SrpRow {
+    uint32_t buf, odd;                   // shared address of the row's entries, offset of the odd columns
+    int q, dir, t;                       // entry of the first pixel's leftmost column at d = 0
+    int sa[2], dhi[2], l[2][3], d[2];    // the lane's two pixels: block sums of A, ranges, the float scores' choice
+    bool close[2];                       // too close to call
+};
+
+// The same for the pixels of a warp together, the blocks of A from its lanes' registers.  64 pairs that are constant along
+// their rows: 1.90 ms (4.96 with the blocks of both images summed for each candidate).
+template <int RHO>
+__device__ __noinline__ int2 srp_settle(uint32_t lo0, uint32_t lo1, uint32_t hi0, uint32_t hi1, const SrpRow &r)
+{
+    constexpr int K = 2 * RHO + 1;
+    uint32_t alo[K + 1], ahi[K + 1];
+    const uint32_t lo[2] = {lo0, lo1}, hi[2] = {hi0, hi1};
+    srp_columns<RHO>(lo, hi, alo, ahi);
+    int out[2];
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+        out[p] = r.d[p];
+        if (!r.close[p])
+            continue;
+        const int l0 = r.l[p][0], l1 = r.l[p][1], l2 = r.l[p][2];
+        SrpBest best;
+        for (int d = max(min(min(l0, l1), l2) - r.t, 0); d <= min(max(max(l0, l1), l2) + r.t, r.dhi[p]); ++d) {
+            if (abs(d - l0) > r.t && abs(d - l1) > r.t && abs(d - l2) > r.t)
+                continue;
+            int N, D;
+            srp_block_nd<RHO>(alo + p, ahi + p, r.sa[p], r.buf, r.odd, r.q + p + (r.dir == 0 ? -d : d), N, D);
+            best.consider(d, N, D);
+        }
+        out[p] = best.d;
+    }
+    return make_int2(out[0], out[1]);
 }
 
 // Layout.  A warp owns a strip of 64 image columns, two adjacent ones per lane, and the 64 - 2 rho pixels
@@ -198,8 +281,8 @@ __device__ __noinline__ int srp_exact_best(const uint8_t *A, const uint8_t *B, i
 // N and D fit 32 bits (n^2 255^2 < 2^28).  The score N / sqrt(D_B) is a float: the conversions, the product
 // and rsqrt.approx (relative error 2^-22.9) err by less than 2^-21 together, so when the best score leads
 // the second best by more than 2^-20 (|s1| + |s2|) the best candidate is the exact one; otherwise the pixel's
-// candidates are compared again in integers, from the images (about one pixel in 10^4).  Ascending d and a
-// strict comparison give ties to the smaller disparity.
+// candidates are compared again in integers (SrpBest).  Ascending d and a strict comparison give ties to the
+// smaller disparity.
 //
 // Few pairs leave most SMs idle, so a map's columns are then split over a cluster (CLUSTER): each CTA also
 // computes kSrpHalo pixels beyond its own on either side, which a pixel per row becomes stale (a row reads
@@ -214,7 +297,7 @@ __device__ __noinline__ int srp_exact_best(const uint8_t *A, const uint8_t *B, i
 // latency chain of a row (about 4400 cycles).  At 1242x375, d_max 127: 64 pairs 3.42 -> 1.83 ms, one pair
 // 3.19 -> 0.76 ms, against every pixel forming its own candidates' products with one CTA per map.
 template <int RHO, int NPREP, bool CLUSTER, int WARPS>
-__global__ void __launch_bounds__(32 * WARPS, 1) k_srp(const SrpArgs a)
+__global__ void __launch_bounds__(32 * WARPS, 1) k_srp(const __grid_constant__ SrpArgs a)
 {
     constexpr int S = srp_strip(RHO), K = 2 * RHO + 1, NB = K * K;
     constexpr int kWin = 30;          // disparities of one candidate mask
@@ -516,10 +599,21 @@ __global__ void __launch_bounds__(32 * WARPS, 1) k_srp(const SrpArgs a)
         constexpr float kEps = 2.25f * 9.5367431640625e-07f;   // 2^-20
         const bool close0 = in0 && r0 > __fmaf_rn(fabsf(b0), -kEps, b0);
         const bool close1 = in1 && r1 > __fmaf_rn(fabsf(b1), -kEps, b1);
-        if (close0)
-            d0 = srp_exact_best<RHO>(A, B, W, v, u0, dir == 0 ? -1 : 1, l00, l01, l02, t, dhi0);
-        if (close1)
-            d1 = srp_exact_best<RHO>(A, B, W, v, u0 + 1, dir == 0 ? -1 : 1, l01, l11, l12, t, dhi1);
+        // The instance for few pairs and 7 x 7 blocks is at its register limit and slower with the state of the warp's
+        // form at hand (one pair of 1242 x 375: 902 us, 952 with it); the others are faster with it (64 pairs: 1619 us,
+        // 1705 without; one pair with 5 x 5 blocks: 935 and 1045).
+        if constexpr (WARPS == kSrpFewWarps && RHO == 3) {
+            if (close0)
+                d0 = srp_exact_best<RHO>(a, v, u0, l00, l01, l02, t, dhi0);
+            if (close1)
+                d1 = srp_exact_best<RHO>(a, v, u0 + 1, l01, l11, l12, t, dhi1);
+        } else if (__any_sync(0xffffffffu, close0 || close1)) {
+            const int2 d = srp_settle<RHO>(ac.lo[0], ac.lo[1], ac.hi[0], ac.hi[1],
+                                           SrpRow{buf, odd, q, dir, t, {sa0, sa1}, {dhi0, dhi1},
+                                                  {{l00, l01, l02}, {l01, l11, l12}}, {d0, d1}, {close0, close1}});
+            d0 = d.x;
+            d1 = d.y;
+        }
         if (mine)
             lv[(v & 1) * n_lv + 1 + pair] = (uint32_t)(in0 ? d0 & 0xffff : 0xffff) | ((in1 ? (uint32_t)d1 : 0xffffu) << 16);
         if (st0)
