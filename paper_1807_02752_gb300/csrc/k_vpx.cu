@@ -25,7 +25,7 @@
 //     while the DP warps work;
 //   - columns off the frame are cells that pay an extra penalty per row: a path through one costs more than
 //     the path that stays in the frame's edge column, so they never win and need no test.
-// The ranks go to a per-frame global buffer (L2-resident), a byte per cell with a bit that says whether the
+// The ranks go to global memory (L2-resident; the frame's part of M_1, not yet written), a byte per cell with a bit that says whether the
 // cell holds votes; a row is stored in planes of one word (four cells) per lane, so that every store of a warp
 // is contiguous.  The backtrack walks blocks of 32 rows: the other warps fetch the columns that the next block
 // can reach and turn their ranks into displacements, so that a step of the walk is one shared-memory load and
@@ -85,18 +85,18 @@ __device__ __forceinline__ void sts1(uint32_t a, uint32_t v) { asm volatile("st.
 // What the kernel reads of a frame's parameters and workspace.
 struct VpxArgs {
     int W, H, chi, vote_rho, lambda_x, tau_x, band_literal;
-    int max_w, max_h, pmax;
+    int pmax;
     const FrameState *fs;
     const int32_t *vcount;
     const int16_t *vbins;
-    uint8_t *gbt;
+    int32_t *M1;          // holds the backtrack rows here
     int16_t *path_x, *pts;
     int32_t *npts, *dbg_mx;
 };
 __host__ __device__ inline VpxArgs vpx_args(const KParams &kp, const Work &w)
 {
-    return {kp.W, kp.H, kp.chi, kp.vote_rho, kp.lambda_x, kp.tau_x, kp.band_literal, w.max_w, w.max_h, w.pmax,
-            w.fs, w.vcount, w.vbins, w.gbt, w.path_x, w.pts, w.npts, w.dbg_mx};
+    return {kp.W, kp.H, kp.chi, kp.vote_rho, kp.lambda_x, kp.tau_x, kp.band_literal, w.pmax,
+            w.fs, w.vcount, w.vbins, w.M1, w.path_x, w.pts, w.npts, w.dbg_mx};
 }
 
 // How a row of W cells lies on the DP warps (vpx_plan).
@@ -167,8 +167,12 @@ __device__ __forceinline__ void scatter_delta(const VpxArgs &a, const VpxMem &S,
         add_votes(a, S, f, v + chi + 1, 0, delta, -unit, t0, stride);
 }
 
-// Byte of cell u in a backtrack row of cells-wide lanes: plane (u % cells) / 4 of one word per lane.
+// Byte of cell u in a backtrack row of cells-wide lanes: plane (u % cells) / 4 of one word per lane.  The rows lie in the
+// frame's part of M_1, from its first 16-byte boundary on (k_m1 writes it two stages later).  H rows fit its 4 W H bytes
+// at every width and its layout (16 columns: 32 bytes a row); a narrow frame that shares a launch, and so the layout, with
+// wide ones has a slot of the widest one's size.
 __host__ __device__ constexpr int bt_plane(int W, int cells) { return 4 * (((W + cells - 1) / cells + 3) & ~3); }
+__host__ __device__ constexpr int bt_row(int W, int cells) { return bt_plane(W, cells) * (cells / 4); }
 __device__ __forceinline__ int bt_byte(int u, int cells, int plane)
 {
     const int g = u / cells, x = u - g * cells;
@@ -261,7 +265,7 @@ struct DpRow {
 template <int TAU, int C, bool LOOK>
 __device__ __forceinline__ int vpx_forward(const VpxArgs &a, const VpxMem &S, const VpxPlan &P, int f, int vtop, uint8_t *gbt)
 {
-    const int W = a.W, vmax = a.H - 1, RB = vpx_row_bytes(W);
+    const int W = a.W, vmax = a.H - 1, RB = bt_row(W, C);
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
     const int R = P.rows, HL = P.halo, HC = HL * C, stride = P.stride;
     const bool dp = warp < P.warps;
@@ -470,7 +474,7 @@ __device__ __noinline__ int vpx_forward_look(const VpxArgs a, const VpxMem S, co
 __device__ __noinline__ int vpx_forward_wide(const VpxArgs a, const VpxMem S, const VpxPlan P, int f,
                                              int vtop, uint8_t *gbt)
 {
-    const int W = a.W, vmax = a.H - 1, RB = vpx_row_bytes(W), tau = a.tau_x;
+    const int W = a.W, vmax = a.H - 1, RB = bt_row(W, P.cells), tau = a.tau_x;
     const int tid = threadIdx.x, nt = blockDim.x, HC = P.halo * P.cells;
     const int plane = bt_plane(W, P.cells);
     int *Ep = S.ring + HC, *Ec = Ep + P.stride, *band = Ec + P.stride, *delta = band + P.stride;
@@ -529,7 +533,7 @@ template <int TAU, int C>
 __device__ __forceinline__ void vpx_dp_body(const VpxArgs &a, const VpxPlan &P, const int f)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int W = a.W, H = a.H, RB = vpx_row_bytes(W);
+    const int W = a.W, H = a.H, RB = bt_row(W, C);
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
     const FrameState fs0 = a.fs[f];
     if (fs0.flags & LD_F_NO_LANES)
@@ -547,7 +551,7 @@ __device__ __forceinline__ void vpx_dp_body(const VpxArgs &a, const VpxPlan &P, 
     S.pid = carve<int16_t>(p, H);
     S.box = carve<int>(p, (size_t)2 * P.warps * 2 * P.halo * C);
     S.ring = carve<int>(p, 0);
-    uint8_t *gbt = a.gbt + (size_t)f * a.max_h * vpx_row_bytes(a.max_w);
+    uint8_t *gbt = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(a.M1 + (size_t)f * H * W) + 15) & ~(uintptr_t)15);
 
     // ---- votes per row of [vtop, vmax], and their total ----
     int votes = 0;

@@ -401,7 +401,6 @@ ld::Work work_from(const ld::Work &w, const ld::KParams &kp, int f0)
     v.inl_x += f * H;
     v.pts += f * 2 * 3 * (size_t)w.pmax;
     v.npts += f * 2;
-    v.gbt += f * (size_t)w.max_h * ld::vpx_row_bytes(w.max_w);
     v.M1 += f * H * W;
     if (v.med)
         v.med += f * H * W;
@@ -830,7 +829,7 @@ int ld_create(const ld_params *p, int32_t max_w, int32_t max_h, int32_t max_batc
     const size_t o_my = take(n * D * H * 4), o_fs = take(n * sizeof(ld::FrameState)), o_rows = take(n * 3 * H * 4);
     const size_t o_py = take(n * D * 2), o_iy = take(n * D), o_ec = take(n * H * 4), o_ed = take(n * H * W * 8);
     const size_t o_vc = take(n * H * 4), o_vb = take(n * H * W * 2), o_px = take(n * H * 2), o_ix = take(n * H);
-    const size_t o_bt = take(n * H * (size_t)ld::vpx_row_bytes(max_w)), o_m1 = take(n * H * W * 4), o_he = take(n * n_starts * 8);
+    const size_t o_m1 = take(n * H * W * 4), o_he = take(n * n_starts * 8);
     const size_t o_pts = take(n * 2 * 3 * pmax * 2), o_np = take(n * 2 * 4);
     const size_t o_tab = take(sizeof(int32_t) * (ld::kWrEntries + ld::kWgEntries));
     const size_t o_cls = take(sizeof(uint16_t) * ld::kClsTables * 512);
@@ -857,7 +856,6 @@ int ld_create(const ld_params *p, int32_t max_w, int32_t max_h, int32_t max_batc
     w.vbins = (int16_t *)(b + o_vb);
     w.path_x = (int16_t *)(b + o_px);
     w.inl_x = (uint8_t *)(b + o_ix);
-    w.gbt = (uint8_t *)(b + o_bt);
     w.M1 = (int32_t *)(b + o_m1);
     w.med = p->bilateral == 2 ? (uint8_t *)(b + o_med) : nullptr;
     w.HE = (int64_t *)(b + o_he);
@@ -869,8 +867,6 @@ int ld_create(const ld_params *p, int32_t max_w, int32_t max_h, int32_t max_batc
     w.wg = h->d_tables + ld::kWrEntries;
     w.cls_tab = (const uint16_t *)(b + o_cls);
     h->d_fdesc = (ld::FrameDesc *)(b + o_fd);
-    w.max_w = max_w;
-    w.max_h = max_h;
     h->d_disp = (float *)(b + o_d);
     h->d_img = (uint8_t *)(b + o_i);
     h->d_lanes = (ld_lanes *)(b + o_l);

@@ -135,8 +135,7 @@ struct Work {
     uint8_t *inl_x;      // [n][H]
     int16_t *pts;        // [n][2][3][pmax] DP path points with data (x, y, index) for the beta / gamma fits
     int32_t *npts;       // [n][2]
-    uint8_t *gbt;        // [n][max_h][vpx_row_bytes(max_w)] V_px backtrack rows
-    int32_t *M1;         // [n][H][W]
+    int32_t *M1;         // [n][H][W]; before it, the V_px backtrack rows
     int32_t *xsum;       // [n][ceil(H/4)][ceil(W/4)] block sums of |G_x w_g| for the learned proposal, or null
     uint8_t *med;        // [n][H][W] median-filtered image (bilateral = 2), or null
     int64_t *HE;         // [n][n_starts]
@@ -145,7 +144,7 @@ struct Work {
     const int32_t *wr;   // [kWrEntries] Q15
     const int32_t *wg;   // [kWgEntries] Q12
     const uint16_t *cls_tab;  // [kClsTables][512] Q15 bilateral weights by distance class and |dI| (zero from 256 on)
-    int32_t max_w, max_h, pmax;
+    int32_t pmax;
 };
 
 // One frame of a call over frames of several sizes (ld_detect_mixed): its own parameters (W, H, start
@@ -187,10 +186,6 @@ __device__ __forceinline__ double i128_to_f64(__int128 x)
     const unsigned int r = (unsigned int)(x & (__int128)0xffffffffu);
     return __dadd_rn(__dmul_rn((double)q, 4294967296.0), (double)r);
 }
-
-// Bytes of one V_px backtrack row: a byte per cell, lanes of at most 20 cells rounded up to four, padded to 16
-// bytes.
-__host__ __device__ inline int vpx_row_bytes(int W) { return (W + 80 + 15) & ~15; }
 
 __device__ __forceinline__ float pow2f(int k) { return __int_as_float((127 + k) << 23); }
 

@@ -17,7 +17,7 @@ constexpr int kDevices = 2, kOptin = 232448, kDefault = 48 * 1024;
 int g_device = 0;
 std::map<const void *, std::string> g_name;
 std::map<std::pair<int, const void *>, int> g_limit;   // (device, kernel): dynamic shared memory allowed
-long long g_launches = 0, g_refused = 0, g_lowered = 0;
+long long g_launches = 0, g_refused = 0, g_lowered = 0, g_allocated = 0;
 std::string g_first_refused, g_first_lowered;
 cudaError_t g_last = cudaSuccess;
 
@@ -54,6 +54,7 @@ void fake_set_device(int d) { g_device = d; }
 long long fake_launches() { return g_launches; }
 long long fake_refused() { return g_refused; }
 long long fake_lowered() { return g_lowered; }
+long long fake_allocated() { return g_allocated; }
 const char *fake_first_refused() { return g_first_refused.c_str(); }
 const char *fake_first_lowered() { return g_first_lowered.c_str(); }
 
@@ -121,9 +122,13 @@ cudaError_t cudaGetLastError()
     g_last = cudaSuccess;
     return e;
 }
-cudaError_t cudaMalloc(void **p, size_t n) { return (*p = std::calloc(n ? n : 1, 1)) ? cudaSuccess : cudaErrorMemoryAllocation; }
-cudaError_t cudaMallocHost(void **p, size_t n) { return cudaMalloc(p, n); }
-cudaError_t cudaHostAlloc(void **p, size_t n, unsigned) { return cudaMalloc(p, n); }
+cudaError_t cudaMallocHost(void **p, size_t n) { return (*p = std::calloc(n ? n : 1, 1)) ? cudaSuccess : cudaErrorMemoryAllocation; }
+cudaError_t cudaHostAlloc(void **p, size_t n, unsigned) { return cudaMallocHost(p, n); }
+cudaError_t cudaMalloc(void **p, size_t n)
+{
+    g_allocated += (long long)n;
+    return cudaMallocHost(p, n);
+}
 cudaError_t cudaFree(void *p)
 {
     std::free(p);
