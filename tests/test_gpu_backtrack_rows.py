@@ -9,16 +9,6 @@ from paper_1807_02752_gb300 import ld, scenes
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def torch_cuda():
-    torch = pytest.importorskip("torch")
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_1807_02752_gb300 import build
-    build.build()
-    return torch
-
-
 def _frame(w, h, seed):
     disp, _ = scenes.make_tiny_frame(w, h, 16, seed)
     return disp, np.random.default_rng([w, h, seed]).integers(0, 256, (h, w), dtype=np.uint8)

@@ -9,16 +9,6 @@ from paper_1807_02752_gb300 import ld, scenes
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def torch_cuda():
-    torch = pytest.importorskip("torch")
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_1807_02752_gb300 import build
-    build.build()
-    return torch
-
-
 @pytest.mark.parametrize("w,h,rho", [(1242, 121, 3), (777, 97, 1), (1613, 64, 2)])
 def test_cluster_exchange_equals_whole_maps(torch_cuda, w, h, rho):
     """One pair, whose maps are split over clusters that exchange their edge estimates every eight rows (a store per

@@ -10,16 +10,6 @@ from paper_1807_02752_gb300 import ld
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def torch_cuda():
-    torch = pytest.importorskip("torch")
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_1807_02752_gb300 import build
-    build.build()
-    return torch
-
-
 def _pair(rng, w, h, kind):
     rows = (np.arange(h) * 7 % 251).astype(np.uint8)[:, None]
     if kind == "rows":            # every candidate of a pixel has the same N and D

@@ -13,16 +13,6 @@ from paper_1807_02752_gb300 import ld, scenes
 LIMIT = 2 ** 26 - 2 ** 16      # energy of a path at which the packed rows end
 
 
-@pytest.fixture(scope="module")
-def torch_cuda():
-    torch = pytest.importorskip("torch")
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_1807_02752_gb300 import build
-    build.build()
-    return torch
-
-
 def _radial(period, w=120, h=1088, d=256, h0=30):
     """A flat road to row h0 whose texture is constant along the lines through one point on the horizon."""
     v, u = np.arange(h)[:, None], np.arange(w)[None, :]
