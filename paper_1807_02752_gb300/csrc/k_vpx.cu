@@ -10,7 +10,7 @@
 //
 // The rows follow one another, so the time is rows x (time of a row), and a row is bound by integer
 // instructions (two cycles each per scheduler) and by its chain of latencies.  Layout:
-//   - four DP warps (eight past 2240 columns), one per scheduler, hold the row in registers, kCells adjacent
+//   - four DP warps (eight past 2400 columns, 2560 with tau_x = 0), one per scheduler, hold the row in registers, kCells adjacent
 //     cells per lane.  A warp's range overlaps its neighbours' by `halo` lanes on each side: a row spoils
 //     tau_x cells at either end, so `rows` rows pass before the warps exchange their edge cells through
 //     shared memory and meet at a barrier (instead of one barrier and a shared-memory window per row);
@@ -763,8 +763,10 @@ cudaError_t launch(const KParams &shape, const VpxArgs &a, const FrameDesc *fd, 
 
 }  // namespace
 
-// Frames a handle accepts: the kernel's shared memory must hold a row of backtrack and the column bitmaps.
-// This bound (four rows of cells, 12288 votes, the per-row arrays, then the bitmaps) is part of ld_create's contract.
+// Frames a handle accepts: a limit on the frame size and the band height that is part of ld_create's contract (it is what a
+// kernel with the votes staged and column bitmaps of the band in shared memory needs: four rows of cells, 12288 votes,
+// the per-row arrays, then the bitmaps).  k_vpx_dp needs less: the ring of any layout is at most kRingBytes or five rows,
+// beside it are 7 H bytes, the edge cells and the backtrack's block list.
 bool vpx_admits(const KParams &kp, size_t budget)
 {
     const size_t H = kp.H, cells = (size_t)(kp.W + 1) / 2 * 2;
@@ -782,7 +784,8 @@ bool vpx_admits(const KParams &kp, size_t budget)
     add(2 * H);
     add(16 * H);
     const size_t fixed = ((s + 15) & ~(size_t)15) + 64;
-    return budget > fixed + (size_t)4 * kp.W * ((32 + 2 * kp.chi + 32 + 31) / 32 + 1);
+    const size_t needed = kRingBytes + 7 * (H + 16) + 4 * (kMaxChunks + 64) + 4 * 2 * 8 * 2 * 10 * kMaxCells;
+    return budget > fixed + (size_t)4 * kp.W * ((32 + 2 * kp.chi + 32 + 31) / 32 + 1) && budget > needed;
 }
 
 // The instances a handle with this tau_x can launch.

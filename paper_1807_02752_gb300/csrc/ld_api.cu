@@ -804,7 +804,7 @@ int ld_create(const ld_params *p, int32_t max_w, int32_t max_h, int32_t max_batc
     }
     build_tables(h->p, h->ws_q, nullptr, nullptr);
 
-    // the V_px DP needs shared memory for a block of backtrack rows and the vote bitmaps of the largest frame
+    // the size limit of the V_px DP and the road DP's shared memory
     ld::KParams kmax = make_kparams(h, max_w, max_h, max_batch);
     if (!ld::vpx_admits(kmax, (size_t)h->smem_optin - 1024) || ld::road_smem_bytes(kmax) > (size_t)h->smem_optin - 1024) {
         delete h;
