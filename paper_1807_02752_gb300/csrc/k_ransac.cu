@@ -415,8 +415,11 @@ __device__ __forceinline__ void fit_body(const KParams &kp, const Work &w, const
         if (LD_IN(pid[j], n_inl, CK_FIT_ROW))
             inl[pid[j]] = 1;
     // final least squares over the remaining set: exact sums (sum t^k for k <= 2M-2, then sum y t^k for k < M),
-    // then the normal equations solved on one warp.  |t| < 2^10, y < 2^13 and at most 2^11 points: sums of t^k
-    // up to k = 5 and of y t^k up to k = 4 fit 64 bits; t^6 .. t^8 are summed as 2^32 hi + lo.
+    // then the normal equations solved on one warp.  |t| <= LD_MAX_H / 2, y < LD_MAX_W and at most LD_MAX_H points: sums
+    // of t^k up to k = 5 and of y t^k up to k = 4 fit 64 bits; t^6 .. t^8 are summed as 2^32 hi + lo.
+    constexpr double kT = LD_MAX_H / 2, kT4 = kT * kT * kT * kT;
+    static_assert(LD_MAX_D <= LD_MAX_H && LD_MAX_H * LD_MAX_W * kT4 < 9.2e18 && LD_MAX_H * kT4 * kT < 9.2e18 &&
+                      LD_MAX_H * kT4 * kT4 / 4294967296.0 < 9.2e18, "exact sums");
     if (!(fl & 2)) {
         constexpr int N64 = 2 * M - 1 > 6 ? 6 : 2 * M - 1;   // powers 0 .. N64 - 1 in 64 bits
         constexpr int NHI = 2 * M - 1 - N64;

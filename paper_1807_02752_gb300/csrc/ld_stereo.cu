@@ -273,7 +273,7 @@ __device__ __noinline__ int2 srp_settle(uint32_t lo0, uint32_t lo1, uint32_t hi0
 // disparity d give the block products P of all its pixels through three shuffles, instead of 2 rho + 1
 // column products per pixel and candidate: neighbouring pixels mostly search the same few disparities (the
 // rows of the synthetic pairs need 6 to 10 distinct ones per strip and row, and 3.3 to 3.8 per pixel), so
-// the warp walks the union of its pixels' search ranges, 32 disparities at a time as a bit mask, and each
+// the warp walks the union of its pixels' search ranges, 30 disparities at a time as a bit mask, and each
 // pixel takes part at its own candidates.  A lane keeps its columns of image A and their sums in registers
 // (the window moves up a row by a byte shift) and publishes the same of image B in shared memory, one
 // 16-byte entry per column {rows 0-3, rows 4-6, s_B, 1 / sqrt(D_B)}, even and odd columns apart so that a
@@ -294,8 +294,9 @@ __device__ __noinline__ int2 srp_settle(uint32_t lo0, uint32_t lo1, uint32_t hi0
 //
 // What bounds it: the rows follow one another (369 at 1242x375).  One CTA per map: the ALU pipe (two cycles
 // per integer instruction) and the wait for the strip with the most distinct disparities.  Clusters: the
-// latency chain of a row (about 4400 cycles).  At 1242x375, d_max 127: 64 pairs 3.42 -> 1.83 ms, one pair
-// 3.19 -> 0.76 ms, against every pixel forming its own candidates' products with one CTA per map.
+// latency chain of a row (about 4400 cycles).  At 1242x375, d_max 127: 64 pairs 3.42 -> 1.57 ms, one pair
+// 3.19 -> 0.77 to 0.90 ms by its texture, against every pixel forming its own candidates' products with one CTA
+// per map.
 template <int RHO, int NPREP, bool CLUSTER, int WARPS>
 __global__ void __launch_bounds__(32 * WARPS, 1) k_srp(const __grid_constant__ SrpArgs a)
 {
@@ -694,8 +695,8 @@ inline SrpShape srp_shape_of(int W, int rho, int dmax, int ctas)
     s.smem = ent + 2 * 4 * (size_t)(s.strips * (S / 2) + 2) + 2 * 4 * kSrpHalo + 6 * 4 * 32 * (size_t)s.strips;
     return s;
 }
-// One CTA per map fills the GPU from about 76 maps on (38 pairs); one pair takes 1.52 ms that way and 0.84 ms on
-// two clusters of 8.  So below that number a map is split over the largest
+// One CTA per map fills the GPU from about 76 maps on (38 pairs); one pair takes 1.57 ms that way and 0.89 ms on
+// two clusters of 8 (1242 x 375).  So below that number a map is split over the largest
 // cluster whose CTAs still find an SM each, every one keeping at least 96 pixels.  Frames wider than a CTA's
 // warps hold are always split.
 inline bool srp_fits(const SrpShape &s) { return s.warps <= kSrpMaxWarps && s.prep <= kSrpPrep; }
