@@ -470,20 +470,24 @@ __device__ __noinline__ int vpx_forward_look(const VpxArgs a, const VpxMem S, co
 
 // The same with plain energies, for a frame whose best path gathers more than 2^26 - 2^16 (67 million; 1242 x 375 pixels
 // with the default parameters cannot hold that much, 1920 x 1080 only if two thirds of all pixels vote for the path's
-// columns): rows in shared memory, compare-select in tie order, two barriers a row, after the packed form in vain.
-__device__ __noinline__ int vpx_forward_wide(const VpxArgs a, const VpxMem S, const VpxPlan P, int f,
-                                             int vtop, uint8_t *gbt)
+// columns): rows in shared memory (five of the ring's), compare-select in tie order, a barrier a row, after the packed form
+// in vain.  A frame of 120 x 1088 whose votes all converge: 1.43 ms in all (1.63 with a run-time tau_x and two barriers a
+// row), 0.37 when its keys fit.
+template <int TAU>
+__device__ __noinline__ int vpx_forward_wide(const VpxArgs a, const VpxMem S, const VpxPlan P, int f, int vtop, uint8_t *gbt)
 {
-    const int W = a.W, vmax = a.H - 1, RB = bt_row(W, P.cells), tau = a.tau_x;
+    const int W = a.W, vmax = a.H - 1, RB = bt_row(W, P.cells), lambda = a.lambda_x;
     const int tid = threadIdx.x, nt = blockDim.x, HC = P.halo * P.cells;
     const int plane = bt_plane(W, P.cells);
-    int *Ep = S.ring + HC, *Ec = Ep + P.stride, *band = Ec + P.stride, *delta = band + P.stride;
+    int *Ep = S.ring + HC, *Ec = Ep + P.stride, *band = Ec + P.stride, *delta = band + P.stride;   // delta: two rows in turn
     for (int u = tid; u < W; u += nt)
-        band[u] = delta[u] = 0;
+        band[u] = delta[u] = delta[P.stride + u] = 0;
     __syncthreads();
     const int r0 = a.band_literal ? vmax : max(vtop, vmax - a.chi);
     for (int r = r0; r <= vmax; ++r)
         add_votes(a, S, f, r, 0, sa(band), 1, tid, nt);
+    if (vmax > vtop)
+        scatter_delta(a, S, f, vmax - 1, vtop, sa(delta + ((vmax - 1) & 1) * P.stride), 1, tid, nt);
     __syncthreads();
     for (int u = tid; u < W; u += nt) {
         Ep[u] = -a.vote_rho * band[u];
@@ -493,27 +497,28 @@ __device__ __noinline__ int vpx_forward_wide(const VpxArgs a, const VpxMem S, co
     }
     __syncthreads();
     for (int v = vmax - 1; v >= vtop; --v) {
-        scatter_delta(a, S, f, v, vtop, sa(delta), 1, tid, nt);
-        __syncthreads();
+        if (v > vtop)   // the next row's changes, while this row is formed
+            scatter_delta(a, S, f, v - 1, vtop, sa(delta + ((v - 1) & 1) * P.stride), 1, tid, nt);
+        int *dv = delta + (v & 1) * P.stride;
         uint8_t *row = gbt + (size_t)v * RB;
         for (int u = tid; u < W; u += nt) {
             int best = Ep[u], arg = 0;
-            for (int k = 1; k <= 2 * tau; ++k) {
-                const int t = (k & 1) ? -((k + 1) >> 1) : (k >> 1);
+#pragma unroll
+            for (int k = 1; k <= 2 * TAU; ++k) {
+                const int d = (k + 1) >> 1, t = (k & 1) ? -d : d;
                 if (u + t < 0 || u + t >= W)
                     continue;
-                const int cand = Ep[u + t] + a.lambda_x * (t < 0 ? -t : t);
-                if (cand < best) {
-                    best = cand;
-                    arg = k;
-                }
+                const int cand = Ep[u + t] + lambda * d;
+                arg = cand < best ? k : arg;
+                best = min(cand, best);
             }
-            band[u] += delta[u];
-            delta[u] = 0;
-            Ec[u] = best - a.vote_rho * band[u];
-            row[bt_byte(u, P.cells, plane)] = (uint8_t)(arg | (band[u] ? kHasVotes : 0u));
+            const int m = band[u] + dv[u];
+            band[u] = m;
+            dv[u] = 0;
+            Ec[u] = best - a.vote_rho * m;
+            row[bt_byte(u, P.cells, plane)] = (uint8_t)(arg | (m ? kHasVotes : 0u));
             if (a.dbg_mx)
-                a.dbg_mx[((size_t)f * a.H + v) * W + u] = -a.vote_rho * band[u];
+                a.dbg_mx[((size_t)f * a.H + v) * W + u] = -a.vote_rho * m;
         }
         __syncthreads();
         int *t = Ep;
@@ -571,7 +576,7 @@ __device__ __forceinline__ void vpx_dp_body(const VpxArgs &a, const VpxPlan &P, 
     const bool look = 16.0 * a.vote_rho * (2.0 * a.chi + 1.0) * votes >= 2147483648.0 - 1048576.0;
     int ustar = look ? vpx_forward_look<TAU, C>(a, S, P, f, vtop, gbt) : vpx_forward<TAU, C, false>(a, S, P, f, vtop, gbt);
     if (ustar < 0)
-        ustar = vpx_forward_wide(a, S, P, f, vtop, gbt);
+        ustar = vpx_forward_wide<TAU>(a, S, P, f, vtop, gbt);
 
     // ---- backtrack from (ustar, vtop): blocks of kBlock rows.  While lane 0 of warp 0 walks a block, the other
     // warps fetch the columns the next one can reach (2 kBlock rows of tau_x from the current column) and turn
